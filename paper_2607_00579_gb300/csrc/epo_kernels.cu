@@ -415,13 +415,12 @@ __global__ void __launch_bounds__(kPoseThreads) k_poses(StepArgs a, int with_gra
           nn += __shfl_xor_sync(0xffffffffu, nn, o);
           no += __shfl_xor_sync(0xffffffffu, no, o);
         }
-        if (vv && e == 0) {
-          const double deg = 180.0 / 3.14159265358979323846;
-          const double cr = fmin(1.0, fmax(-1.0, (tr - 1.0) * 0.5));
-          a.pose_dR[v] = deg * acos(cr);
-          const double nm = sqrt(nn) * sqrt(no);
-          a.pose_dt[v] = nm > 0.0 ? deg * acos(fmin(1.0, fmax(-1.0, dot / nm))) : 0.0;
-        }
+        // lane 0 takes the rotation's angle, lane 1 the translations': one acos for both
+        const double deg = 180.0 / 3.14159265358979323846;
+        const double nm = sqrt(nn) * sqrt(no);
+        const double cr = e == 0 ? (tr - 1.0) * 0.5 : (nm > 0.0 ? dot / nm : 1.0);
+        const double ang = deg * acos(fmin(1.0, fmax(-1.0, cr)));
+        if (vv && e < 2) (e == 0 ? a.pose_dR : a.pose_dt)[v] = ang;
       }
     }
   } else {
@@ -685,16 +684,89 @@ __global__ void k_round_bf16(const float* src, uint16_t* dst, int64_t n) {
 }
 
 // ------------------------------------------------------------------------------------
-// launchers
+// Block-wide selection, used by the sub-sampling (a cut in the pair keys) and the schedule
+// (order statistics of the pose changes).
+//
+// Finds the k-th smallest (1-based) of the n 64-bit keys key(0) .. key(n - 1) by a radix select,
+// one byte per pass from the top: a 256-bin histogram in shared memory, then one warp scans it
+// (8 bins per lane, a shuffle scan, no serial walk over the bins: with one thread walking them a
+// pass took 3.2 us, 26 us for the sub-sampling's eight passes over 1,200 pairs and ~95 us for the
+// schedule's 32 over 120 views; a step of 120 views, 1,200 pairs and a budget of 500 went from 250
+// to 127 us with this and the rank counting below).  A bin that holds a single key ends the search: its key is read
+// off directly (random 64-bit keys: two or three passes).  Every thread of the block calls it;
+// afterwards sel->prefix is the key, sel->k its rank among the keys equal to it and sel->count
+// how many those are.
 // ------------------------------------------------------------------------------------
+struct BlockSelect {
+  unsigned hist[256];
+  unsigned long long prefix;
+  unsigned k, count;
+};
+
+template <class KeyOf>
+__device__ void block_select(BlockSelect* sel, int n, unsigned k, const KeyOf& key) {
+  __syncthreads();  // the previous selection's results have been read
+  if (threadIdx.x == 0) {
+    sel->prefix = 0ull;
+    sel->k = k;
+  }
+  for (int shift = 56; shift >= 0; shift -= 8) {
+    for (int b = threadIdx.x; b < 256; b += blockDim.x) sel->hist[b] = 0u;
+    __syncthreads();
+    const unsigned long long prefix = sel->prefix;
+    const unsigned long long hm = shift == 56 ? 0ull : (~0ull << (shift + 8));
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const unsigned long long x = key(i);
+      if ((x & hm) == prefix) atomicAdd(&sel->hist[(x >> shift) & 255u], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const unsigned kk = sel->k;  // read by every lane before the shuffles, written after them
+      unsigned c[8], sum = 0u;
+#pragma unroll
+      for (int b = 0; b < 8; ++b) sum += c[b] = sel->hist[8 * threadIdx.x + b];
+      unsigned incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned up = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)threadIdx.x >= o) incl += up;
+      }
+      unsigned cum = incl - sum;
+      if (cum < kk && kk <= incl) {  // the cut lies in this lane's bins
+        int d = -1;
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+          if (d < 0 && kk <= cum + c[b]) {
+            d = b;
+            sel->k = kk - cum;
+            sel->count = c[b];
+          }
+          cum += c[b];
+        }
+        sel->prefix = prefix | ((unsigned long long)(8 * threadIdx.x + d) << shift);
+      }
+    }
+    __syncthreads();
+    if (sel->count == 1u && shift > 0) {  // uniform over the block
+      const unsigned long long top = sel->prefix, tm = ~0ull << shift;
+      __syncthreads();  // every thread has read the prefix
+      for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const unsigned long long x = key(i);
+        if ((x & tm) == top) sel->prefix = x;  // one thread's
+      }
+      break;
+    }
+  }
+  __syncthreads();
+}
+
 // ------------------------------------------------------------------------------------
 // Stochastic viewgraph sub-sampling (Algorithm 3, Appendix A.3): each evaluation uses a
 // fresh uniform random subset of min(P_s, M) of a scene's P_s pairs.  Pair p (index within
 // its scene) at step s gets the key SplitMix64(seed ^ (s << 32 | p)) (the output function of
 // Steele, Lea and Flood's generator, OOPSLA 2014, on state + its golden-ratio increment);
 // the M smallest keys are taken, ties by index.  One block per scene finds the M-th
-// smallest key by a radix select over its 8 bytes (a 256-bin histogram per byte, high byte
-// first), then writes every pair's flag and loss weight.
+// smallest key (block_select), then writes every pair's flag and loss weight.
 // ------------------------------------------------------------------------------------
 __device__ __forceinline__ uint64_t splitmix64_out(uint64_t state) {
   uint64_t z = state + 0x9E3779B97F4A7C15ull;
@@ -710,90 +782,54 @@ __device__ __forceinline__ uint64_t subsample_key(uint64_t seed, int64_t step, i
 constexpr int kSubsampleThreads = 1024;
 
 __global__ void __launch_bounds__(kSubsampleThreads) k_subsample(StepArgs a) {
-  __shared__ unsigned hist[256];
-  __shared__ unsigned long long s_prefix;
-  __shared__ int s_k, s_eq;
+  __shared__ BlockSelect sel;
+  __shared__ double s_w;
   const int sc = blockIdx.x;
   const int off = a.scene_pair_off[sc], P = a.scene_pair_off[sc + 1] - off;
   const int M = a.pair_budget;
   const int64_t step = *a.step;
   const uint64_t seed = a.subsample_seed;
   const bool all = M <= 0 || P <= M;
-  const int na = all ? P : M;
+  // one FP64 division per block (one per pair held the FP64 pipe for longer than the selection)
+  if (threadIdx.x == blockDim.x - 1) s_w = 2.0 / (all ? P : M);
   uint64_t thr = ~0ull;
-  int k_eq = 0;
   if (!all) {
-    if (threadIdx.x == 0) {
-      s_prefix = 0ull;
-      s_k = M;  // rank (1-based) of the cut within the keys that share the prefix
-    }
-    for (int shift = 56; shift >= 0; shift -= 8) {
-      for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0u;
-      __syncthreads();
-      const uint64_t prefix = s_prefix;
-      const uint64_t hm = shift == 56 ? 0ull : (~0ull << (shift + 8));
-      for (int p = threadIdx.x; p < P; p += blockDim.x) {
-        const uint64_t key = subsample_key(seed, step, p);
-        if ((key & hm) == (prefix & hm)) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        const unsigned k = (unsigned)s_k;
-        unsigned cum = 0u;
-        int d = 0;
-        for (; d < 255; ++d) {
-          if (cum + hist[d] >= k) break;
-          cum += hist[d];
-        }
-        s_k = (int)(k - cum);
-        s_prefix = prefix | ((uint64_t)d << shift);
-      }
-      __syncthreads();
-    }
-    thr = s_prefix;  // the M-th smallest key
-    k_eq = s_k;      // how many of the keys equal to it are taken
-    if (threadIdx.x == 0) s_eq = 0;
-    __syncthreads();
-    for (int p = threadIdx.x; p < P; p += blockDim.x)
-      if (subsample_key(seed, step, p) == thr) atomicAdd(&s_eq, 1);
+    block_select(&sel, P, (unsigned)M, [&](int p) { return subsample_key(seed, step, p); });
+    thr = sel.prefix;  // the M-th smallest key
+  } else {
     __syncthreads();
   }
-  const bool ties = !all && s_eq != k_eq;  // equal 64-bit keys across the cut: index order decides
+  const double w2 = s_w;
+  const int k_eq = all ? 0 : (int)sel.k;                // how many of the keys equal to it are taken
+  const bool ties = !all && (int)sel.count != k_eq;  // equal 64-bit keys across the cut: index order decides
+  const auto weight = [&](int q, bool act) {
+    double w = 0.0;
+    if (act) {
+      w = w2;
+      if (a.norm_all) {
+        const int32_t n = a.views[a.pair_src[q]].n_rec;
+        w = n > 0 ? w / (double)n : 0.0;
+      }
+    }
+    return w;
+  };
   for (int p = threadIdx.x; p < P; p += blockDim.x) {
     bool act = true;
     if (!all) {
       const uint64_t key = subsample_key(seed, step, p);
       act = key < thr || (key == thr && !ties);
     }
-    const int q = off + p;
-    double w = 0.0;
-    if (act) {
-      w = 2.0 / na;
-      if (a.norm_all) {
-        const int32_t n = a.views[a.pair_src[q]].n_rec;
-        w = n > 0 ? w / (double)n : 0.0;
-      }
-    }
-    a.pair_active_w[q] = act ? 1 : 0;
-    a.pair_lw[q] = w;
+    a.pair_active_w[off + p] = act ? 1 : 0;
+    a.pair_lw[off + p] = weight(off + p, act);
   }
   __syncthreads();  // every flag is written before the tied ones are set in index order
   if (ties && threadIdx.x == 0) {
     int taken = 0;
     for (int p = 0; p < P; ++p)
       if (subsample_key(seed, step, p) == thr) {
-        const int q = off + p;
         const bool act = taken++ < k_eq;
-        double w = 0.0;
-        if (act) {
-          w = 2.0 / na;
-          if (a.norm_all) {
-            const int32_t n = a.views[a.pair_src[q]].n_rec;
-            w = n > 0 ? w / (double)n : 0.0;
-          }
-        }
-        a.pair_active_w[q] = act ? 1 : 0;
-        a.pair_lw[q] = w;
+        a.pair_active_w[off + p] = act ? 1 : 0;
+        a.pair_lw[off + p] = weight(off + p, act);
       }
   }
 }
@@ -802,65 +838,68 @@ __global__ void __launch_bounds__(kSubsampleThreads) k_subsample(StepArgs a) {
 // Optimization schedule (Section 3): after every step, theta_95 = max(95th percentile of
 // the rotation changes, 95th percentile of the translation-direction changes) over the
 // scene's poses, then the dual-phase rule.  One block per scene; the percentile takes the
-// two order statistics around 0.95 (n - 1) by radix select over the bit patterns of the
-// (non-negative) doubles and interpolates between them linearly.
+// two order statistics around 0.95 (n - 1) of the (non-negative) doubles, compared by their
+// bit patterns, and interpolates between them linearly.
+//
+// Up to kRankViews views every thread counts the values below its own (both sequences at once:
+// n broadcast reads from shared memory, no passes, no atomics); above, where n^2 compares cost
+// more, block_select finds the lower one and the next is a minimum over the values above it.
 // ------------------------------------------------------------------------------------
 constexpr int kScheduleThreads = 256;
-
-// k-th smallest (0-based) of n non-negative doubles; every thread of the block calls it.
-__device__ double block_kth(const double* x, int n, int k, unsigned* hist, unsigned long long* s_prefix, int* s_k) {
-  if (threadIdx.x == 0) {
-    *s_prefix = 0ull;
-    *s_k = k + 1;
-  }
-  for (int shift = 56; shift >= 0; shift -= 8) {
-    for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0u;
-    __syncthreads();
-    const unsigned long long prefix = *s_prefix;
-    const unsigned long long hm = shift == 56 ? 0ull : (~0ull << (shift + 8));
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const unsigned long long key = (unsigned long long)__double_as_longlong(x[i]);
-      if ((key & hm) == (prefix & hm)) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const unsigned kk = (unsigned)*s_k;
-      unsigned cum = 0u;
-      int d = 0;
-      for (; d < 255; ++d) {
-        if (cum + hist[d] >= kk) break;
-        cum += hist[d];
-      }
-      *s_k = (int)(kk - cum);
-      *s_prefix = prefix | ((unsigned long long)d << shift);
-    }
-    __syncthreads();
-  }
-  return __longlong_as_double((long long)*s_prefix);
-}
-
-__device__ double block_percentile95(const double* x, int n, unsigned* hist, unsigned long long* s_prefix, int* s_k) {
-  if (n <= 0) return 0.0;
-  const double pos = 0.95 * (double)(n - 1);
-  const int lo = (int)floor(pos);
-  const double a = block_kth(x, n, lo, hist, s_prefix, s_k);
-  if (lo >= n - 1) return a;
-  const double b = block_kth(x, n, lo + 1, hist, s_prefix, s_k);
-  return a + (b - a) * (pos - (double)lo);
-}
+constexpr int kRankViews = 256;
 
 __global__ void __launch_bounds__(kScheduleThreads) k_schedule(StepArgs a) {
-  __shared__ unsigned hist[256];
-  __shared__ unsigned long long s_prefix;
-  __shared__ int s_k;
+  __shared__ BlockSelect sel;
+  __shared__ unsigned long long s_key[2][kRankViews];
+  __shared__ unsigned long long s_stat[2][2];  // [rotation, translation][lower, next] order statistic
+  __shared__ double s_pct[2];
   const int sc = blockIdx.x;
   const int v0 = a.scene_view_off[sc], n = a.scene_view_off[sc + 1] - v0;
   int32_t* st = a.sched_state + 2 * sc;
   if (st[0] == 3) return;  // uniform over the block: converged earlier
-  const double pR = block_percentile95(a.pose_dR + v0, n, hist, &s_prefix, &s_k);
-  const double pT = block_percentile95(a.pose_dt + v0, n, hist, &s_prefix, &s_k);
+  const unsigned long long* x[2] = {reinterpret_cast<const unsigned long long*>(a.pose_dR + v0),
+                                    reinterpret_cast<const unsigned long long*>(a.pose_dt + v0)};
+  const double pos = 0.95 * (double)(n - 1);
+  const int lo = (int)floor(pos);
+  if (n <= kRankViews) {
+    for (int e = threadIdx.x; e < 2 * n; e += blockDim.x) s_key[e >= n][e >= n ? e - n : e] = x[e >= n][e >= n ? e - n : e];
+    __syncthreads();
+    for (int e = threadIdx.x; e < 2 * n; e += blockDim.x) {
+      const int w = e >= n, i = w ? e - n : e;
+      const unsigned long long key = s_key[w][i];
+      int rank = 0;  // equal values keep their order: the ranks are a permutation
+      for (int j = 0; j < n; ++j) rank += s_key[w][j] < key || (s_key[w][j] == key && j < i);
+      if (rank == lo) s_stat[w][0] = key;
+      if (rank == lo + 1) s_stat[w][1] = key;
+    }
+    __syncthreads();
+  } else {
+    for (int w = 0; w < 2; ++w) {
+      block_select(&sel, n, (unsigned)(lo + 1), [&](int i) { return x[w][i]; });
+      const unsigned long long key = sel.prefix;
+      if (threadIdx.x == 0) {
+        s_stat[w][0] = key;
+        s_stat[w][1] = sel.k < sel.count ? key : ~0ull;  // the next one is equal, or the smallest above
+      }
+      __syncthreads();
+      if (sel.k >= sel.count)
+        for (int i = threadIdx.x; i < n; i += blockDim.x)
+          if (x[w][i] > key) atomicMin(&s_stat[w][1], x[w][i]);
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < 2) {
+    const int w = threadIdx.x;
+    const double p0 = __longlong_as_double((long long)s_stat[w][0]);
+    s_pct[w] = p0;
+    if (lo < n - 1) {
+      const double p1 = __longlong_as_double((long long)s_stat[w][1]);
+      s_pct[w] = p0 + (p1 - p0) * (pos - (double)lo);
+    }
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    const double theta = fmax(pR, pT);
+    const double theta = fmax(s_pct[0], s_pct[1]);
     a.theta95[sc] = theta;
     const int64_t step = *a.step - 1;  // the step just taken (the pose kernel advanced the counter)
     if (st[0] == 1) {
@@ -880,6 +919,9 @@ __global__ void __launch_bounds__(kScheduleThreads) k_schedule(StepArgs a) {
   }
 }
 
+// ------------------------------------------------------------------------------------
+// launchers
+// ------------------------------------------------------------------------------------
 cudaError_t launch_schedule(const StepArgs& a, cudaStream_t s) {
   k_schedule<<<a.n_scenes, kScheduleThreads, 0, s>>>(a);
   return cudaGetLastError();
