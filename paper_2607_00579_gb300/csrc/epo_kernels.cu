@@ -10,7 +10,7 @@
 // Both small kernels are FP64 latency chains on a few warps: they run 32-thread blocks, so
 // that their FP64 work spreads over many SMs (an FP64 warp instruction occupies its
 // sub-partition's FP64 pipe for many cycles on this GPU).
-// Construction helpers: k_edt (exact distance transform field), k_round_bf16, k_map_check.
+// Construction helpers: k_edt_rows, k_edt_cols (exact distance transform field), k_round_bf16, k_map_check.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -637,43 +637,114 @@ __global__ void k_map_check(const void* map, int dtype, int64_t n, int32_t* bad)
   if (cnt) atomicAdd(bad, cnt);
 }
 
-// Exact Euclidean distance transform, one block per strip of CB columns.  Pass 1 puts, for
-// every pixel of the strip, the squared distance to the nearest edge of its own row into
-// shared memory (outward scan of the mask row).  Pass 2 takes, per pixel, the minimum over
-// rows y' of f(x, y') + (y - y')^2, scanning outward from y and stopping once (y - y')^2
-// alone exceeds the best value.  Every value is an integer below 2^24, exact in f32; the
-// final sqrtf is correctly rounded.
-constexpr int kEdtCols = 32;
-constexpr int kEdtMaxH = 1536;  // kEdtCols * kEdtMaxH * 4 B = 192 KB of shared memory
+// Exact Euclidean distance transform in two launches, with the output as the only scratch.
+//
+// Rows (k_edt_rows): f(y, x) = the squared distance to the nearest edge of row y.  One warp per
+// row: the row's bytes become 32-pixel words by ballots (lane c keeps word c of a segment of 1024
+// pixels), two shuffle scans give every word the last edge before it and the first one after it,
+// and each pixel's two neighbours are then bit scans of its own word.  No pixel walks its row.
+// Columns (k_edt_cols): the minimum over rows y' of f(y', x) + (y - y')^2, a strip of kEdtCols
+// columns in shared memory, scanned outward from y until (y - y')^2 alone reaches the best value.
+// Rows past the border are read at the border: their candidate is then no smaller than the border
+// row's own.  Every value is an integer below 2^24 (distances to 4096), exact in f32; the final
+// sqrtf is correctly rounded.
+//
+// Bound by latency: a 518x392 map is 0.2 MB in and 0.8 MB out.  Strips of 4 columns give 130
+// blocks there (strips of 32, with the row walk inside each block, gave 17 blocks and 250-360 us;
+// 16 maps through the public call took 6.1 ms, now 0.25 ms).
+constexpr int kEdtCols = 4;
+constexpr int kEdtMaxH = 1536;
+constexpr int kEdtRowThreads = 64;
+constexpr int kEdtColThreads = 512;
+constexpr int kEdtNone = 0x7fffffff;  // no edge on that side (before a pixel: -1)
 
-__global__ void k_edt(const uint8_t* edges, int W, int H, float* out) {
-  extern __shared__ float f[];  // [H][kEdtCols]
-  const float INF = 3.0e38f;
-  const int xb = blockIdx.x * kEdtCols;
-  const int nc = min(kEdtCols, W - xb);
-  for (int e = threadIdx.x; e < nc * H; e += blockDim.x) {
-    const int c = e % nc, y = e / nc;
-    const int x = xb + c;
-    const uint8_t* row = edges + (size_t)y * W;
-    float best = INF;
-    for (int d = 0; d < W; ++d) {
-      const bool l = x - d >= 0 && row[x - d];
-      const bool r = x + d < W && row[x + d];
-      if (l || r) { best = (float)d * (float)d; break; }
-      if (x - d < 0 && x + d >= W) break;
+__device__ __forceinline__ float edt_square(int d) { return d == kEdtNone ? 3.0e38f : (float)d * (float)d; }
+
+__global__ void __launch_bounds__(kEdtRowThreads) k_edt_rows(const uint8_t* edges, int W, int H, float* out) {
+  griddep_launch_dependents();
+  const int lane = threadIdx.x & 31;
+  const int y = blockIdx.x * (kEdtRowThreads / 32) + (threadIdx.x >> 5);
+  if (y >= H) return;
+  const uint8_t* row = edges + (size_t)y * W;
+  float* o = out + (size_t)y * W;
+  const int nseg = (W - 1) / 1024 + 1;
+  int next = kEdtNone;  // the first edge after the segment
+  for (int s = nseg - 1; s >= 0; --s) {
+    const int xs = s * 1024, left_px = W - xs;
+    const int nw = left_px >= 1024 ? 32 : (left_px + 31) / 32;  // words of the segment
+    unsigned word = 0u;
+    for (int c0 = 0; c0 < nw; c0 += 16) {  // 16 loads in flight
+      unsigned char b[16];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const int k = 32 * (c0 + c) + lane;
+        b[c] = k < left_px ? row[xs + k] : (unsigned char)0;
+      }
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const unsigned m = __ballot_sync(0xffffffffu, b[c] != 0);
+        if (lane == c0 + c) word = m;
+      }
     }
-    f[y * kEdtCols + c] = best;
+    // last edge before the lane's word (within the segment), first edge after it
+    const int x0 = xs + 32 * lane;
+    int last = word ? x0 + 31 - __clz(word) : -1;
+    int first = word ? x0 + __ffs(word) - 1 : kEdtNone;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int l = __shfl_up_sync(0xffffffffu, last, d), f = __shfl_down_sync(0xffffffffu, first, d);
+      if (lane >= d) last = max(last, l);
+      if (lane + d < 32) first = min(first, f);
+    }
+    first = min(first, next);
+    int before = __shfl_up_sync(0xffffffffu, last, 1), after = __shfl_down_sync(0xffffffffu, first, 1);
+    if (lane == 0) before = -1;
+    if (lane == 31) after = next;
+    next = __shfl_sync(0xffffffffu, first, 0);
+    for (int c = 0; c < nw; ++c) {
+      const unsigned w = __shfl_sync(0xffffffffu, word, c);
+      const int lb = __shfl_sync(0xffffffffu, before, c), ra = __shfl_sync(0xffffffffu, after, c);
+      const int x = xs + 32 * c + lane;
+      const unsigned lo = w & ((2u << lane) - 1u), hi = w >> lane;
+      const int l = lo ? xs + 32 * c + 31 - __clz(lo) : lb;
+      const int r = hi ? x + __ffs(hi) - 1 : ra;
+      const int d = min(l < 0 ? kEdtNone : x - l, r == kEdtNone ? kEdtNone : r - x);
+      // rows of several segments: the distance itself, until the edges to the left are known
+      if (x < W) o[x] = nseg == 1 ? edt_square(d) : __int_as_float(d);
+    }
+  }
+  if (nseg == 1) return;
+  int last = -1;  // the last edge so far
+  for (int c = 0; c <= (W - 1) / 32; ++c) {
+    const int k = W - 32 * c, x = 32 * c + lane;  // pixels left from this word on
+    const unsigned m = __ballot_sync(0xffffffffu, lane < k && row[x] != 0);
+    if (lane < k) o[x] = edt_square(min(__float_as_int(o[x]), last < 0 ? kEdtNone : x - last));
+    if (m) last = 32 * c + 31 - __clz(m);
+  }
+}
+
+__global__ void __launch_bounds__(kEdtColThreads) k_edt_cols(int W, int H, float* out) {
+  extern __shared__ float f[];  // [H][kEdtCols]
+  const int xb = blockIdx.x * kEdtCols;
+  griddep_wait();  // the rows' distances
+  for (int e = threadIdx.x; e < kEdtCols * H; e += blockDim.x) {
+    const int x = xb + e % kEdtCols;
+    f[e] = x < W ? out[(size_t)(e / kEdtCols) * W + x] : 0.f;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < nc * H; e += blockDim.x) {
-    const int c = e % nc, y = e / nc;
-    float best = f[y * kEdtCols + c];
-    for (int d = 1; (float)d * (float)d < best && (y - d >= 0 || y + d < H); ++d) {
-      const float dd = (float)d * (float)d;
-      if (y - d >= 0) best = fminf(best, f[(y - d) * kEdtCols + c] + dd);
-      if (y + d < H) best = fminf(best, f[(y + d) * kEdtCols + c] + dd);
+  for (int e = threadIdx.x; e < kEdtCols * H; e += blockDim.x) {
+    const int c = e % kEdtCols, y = e / kEdtCols;
+    if (xb + c >= W) continue;
+    float best = f[e];
+    const int far = max(y, H - 1 - y);
+    for (int d = 1; d <= far && (float)d * (float)d < best; d += 4) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float dd = (float)(d + k) * (float)(d + k);
+        best = fminf(best, fminf(f[max(y - d - k, 0) * kEdtCols + c], f[min(y + d + k, H - 1) * kEdtCols + c]) + dd);
+      }
     }
-    out[(size_t)y * W + xb + c] = best >= INF ? (float)(W + H) : sqrtf(best);
+    out[(size_t)y * W + xb + c] = best >= 3.0e38f ? (float)(W + H) : sqrtf(best);
   }
 }
 
@@ -1043,12 +1114,13 @@ cudaError_t launch_map_check(const void* map, int dtype, int64_t n, int32_t* bad
 int edt_max_height() { return kEdtMaxH; }
 
 cudaError_t launch_edt(const uint8_t* edges, int W, int H, float* map, cudaStream_t s) {
-  const size_t smem = sizeof(float) * kEdtCols * (size_t)H;
-  cudaError_t e = cudaFuncSetAttribute(k_edt, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float) * kEdtCols * kEdtMaxH));
+  constexpr int rows = kEdtRowThreads / 32;
+  k_edt_rows<<<(H + rows - 1) / rows, kEdtRowThreads, 0, s>>>(edges, W, H, map);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_edt<<<(W + kEdtCols - 1) / kEdtCols, 256, smem, s>>>(edges, W, H, map);
-  return cudaGetLastError();
+  // shared memory: 24 KB at the largest H
+  return launch_pdl(k_edt_cols, dim3((W - 1) / kEdtCols + 1), dim3(kEdtColThreads), sizeof(float) * kEdtCols * (size_t)H, s,
+                    W, H, map);
 }
 
 cudaError_t launch_round_bf16(const float* src, uint16_t* dst, int64_t n, cudaStream_t s) {
