@@ -115,7 +115,7 @@ typedef struct {
   double beta1, beta2, adam_eps; /* Adam moments (Section 3: 0.9, 0.999) */
   int32_t autotune;          /* 1: pick the kernel schedule by timing on first use;
                                 2: the same, each timed launch starting from a cold L2 */
-  int32_t gather;            /* EPO_GATHER_* (AUTO = LDG unless autotuned) */
+  int32_t gather;            /* EPO_GATHER_* (AUTO = TEX unless autotuned) */
   int32_t block_threads;     /* 0 = default (256); else 64..512, multiple of 32 */
   int32_t records_per_thread;/* 0 = default (2); 1, 2, 4 or 8 (two in flight at a time;
                                 refine scenes: 2) */

@@ -1,0 +1,56 @@
+"""The default schedule against explicit ones on the same scene.  The sums of a work item are formed
+in one order whatever the gather path and the split of its pairs, so the results agree to the order
+of FP64 atomics (1e-12 leaves four digits for cancellation in the gradient)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("CUDA GPU required", allow_module_level=True)
+
+import paper_2607_00579_gb300 as epo  # noqa: E402
+
+B = epo._binding
+
+
+def scene(W, H, n_views, n_rec, k, mixed, **opt):
+    r = np.random.default_rng([W, H, n_views])
+    rec = np.zeros((n_rec * n_views, 4), np.float32)
+    rec[:, 0], rec[:, 1] = r.integers(0, W, len(rec)), r.integers(0, H, len(rec))
+    rec[:, 2] = np.float16(r.uniform(2, 5, len(rec)))
+    maps = [r.uniform(0, 12, (H, W)).astype(np.float32).view(np.uint32) & 0xffff0000 for _ in range(n_views)]
+    maps = [m.astype(np.uint32).view(np.float32) for m in maps]
+    T = np.tile(np.eye(3, 4).reshape(-1), (n_views, 1))
+    T[:, [3, 7, 11]] = r.normal(0, 0.1, (n_views, 3))
+    kw = {}
+    if mixed:
+        packed = np.zeros((len(rec), 4), np.uint16)
+        packed[:, :2], packed[:, 2] = rec[:, :2], rec[:, 2].astype(np.float16).view(np.uint16)
+        rec, maps = packed, [(m.view(np.uint32) >> 16).astype(np.uint16) for m in maps]
+        kw = dict(record_dtype=epo.EPO_F16, map_dtype=epo.EPO_BF16)
+    pairs = np.array([(i, (i + 1 + j) % n_views) for i in range(n_views) for j in range(k)], np.int32)
+    s = epo.Scene.single(np.full(n_views, W), np.full(n_views, H), np.tile([W, W, (W - 1) / 2, (H - 1) / 2], (n_views, 1)),
+                         n_rec * np.arange(n_views + 1), rec, maps, pairs, options=epo.default_options(**opt), **kw)
+    s.set_poses(T)
+    return s
+
+
+def evaluate(s, refine):
+    if refine:
+        i = s.info()
+        return B.epo_refine_loss_and_grad(s.handle, i.n_scenes, i.n_views, i.n_records)
+    return (*s.loss_and_grad(), s.pair_stats())
+
+
+@pytest.mark.parametrize("W,H,n_views,n_rec,k", [(2, 2, 2, 9, 1), (3, 65, 3, 700, 2), (64, 48, 5, 513, 4),
+                                                 (161, 123, 12, 1500, 11), (97, 80, 40, 5000, 8)])
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("refine", [0, 1])
+def test_default_equals_plain_loads(W, H, n_views, n_rec, k, mixed, refine):
+    a = scene(W, H, n_views, n_rec, k, mixed, refine=refine)
+    b = scene(W, H, n_views, n_rec, k, mixed, refine=refine, gather=epo.EPO_GATHER_LDG, tail_pairs=0)
+    assert (a.info().gather, b.info().gather) == (epo.EPO_GATHER_TEX, epo.EPO_GATHER_LDG)
+    for x, y in zip(evaluate(a, refine), evaluate(b, refine)):
+        assert np.abs(x - y).max() <= 1e-12 * max(np.abs(y).max(), 1e-300)
