@@ -6,9 +6,12 @@
 // cameras, inside view j, and returns within tau pixels.  A pair is kept when the fraction
 // is at least min_frac in both directions (the paper's 12.5 % at tau = 3 px).
 //
-// One block per ordered pair, FP64 throughout (the construction is run once; ~100 FP64
-// operations per grid pixel), with every product and sum rounded on its own in a fixed
-// order, so the counts do not depend on how the compiler would fuse them.
+// The counts are those of an FP64 evaluation in which every product, sum, quotient and root is
+// rounded on its own in a fixed order (trip_exact), whatever the compiler would fuse.  On this GPU
+// that evaluation is ~200 instructions of the 1/64-rate FP64 pipe per grid pixel (24 views of
+// 518x392 at stride 4: 2.5 ms), so every grid pixel first runs in FP32 beside a bound on its error,
+// and only those with a decision inside the bound (well under 1 % of them) are kept in shared
+// memory and evaluated in FP64, 32 to a warp (the same 24 views: 2544 -> 205 us for the whole call).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -50,48 +53,206 @@ __device__ bool reproject(const VgView& v, const VgView& w, double x, double y, 
   return true;
 }
 
-constexpr int kVgThreads = 256;
+// One round trip of pixel (x, y) of view i at depth z, in FP64.
+__device__ __noinline__ bool trip_exact(const VgView& vi, const VgView& vj, const float* depth, int x, int y, float zf,
+                                        double tau) {
+  const double z = (double)zf;
+  double xj, yj;
+  if (!reproject(vi, vj, (double)x, (double)y, z, xj, yj)) return false;
+  if (!(xj >= 0.0 && xj <= (double)(vj.W - 1) && yj >= 0.0 && yj <= (double)(vj.H - 1))) return false;
+  const int xn = (int)floor(add(xj, 0.5)), yn = (int)floor(add(yj, 0.5));  // nearest pixel
+  if (xn < 0 || xn >= vj.W || yn < 0 || yn >= vj.H) return false;
+  const double zj = (double)depth[vj.off + (int64_t)yn * vj.W + xn];
+  if (!(zj > 0.0) || !isfinite(zj)) return false;
+  double xb, yb;
+  if (!reproject(vj, vi, xj, yj, zj, xb, yb)) return false;
+  const double dx = sub(xb, (double)x), dy = sub(yb, (double)y);
+  return __dsqrt_rn(add(mul(dx, dx), mul(dy, dy))) < tau;
+}
 
-__global__ void __launch_bounds__(kVgThreads) k_viewgraph(const VgView* views, const float* depth, int n, int stride,
-                                                          double tau, double* frac) {
-  const int i = blockIdx.x / n, j = blockIdx.x % n;
-  if (i == j) {
-    if (threadIdx.x == 0) frac[blockIdx.x] = 0.0;
-    return;  // uniform over the block
+constexpr int kVgThreads = 256;
+constexpr int kVgExact = 1024;   // grid pixels a block keeps for the FP64 evaluation
+constexpr int kVgBlocks = 8 * 152;  // one wave of resident blocks: fewer pairs are split over several
+
+// One direction of a pair in FP32: Y = M X + t, and the constants of the bound
+//   |Y_r - Y_r(FP64)| <= E = z Ca + Cb.
+// With u = 2^-24 and G >= 1, |X0| / z, |X1| / z anywhere in the image: X0 = ((x - cx) / fx) z carries
+// 5u G z (the rounded cx, 1 / fx, and three operations), M's and t's entries u, the FMA chain at
+// most 3u of each term, so |dY_r| <= 9u sum_c |M_rc| G z + 4u |t_r|: Ca = 10u m G, Cb = 10u max |t|
+// with m the largest row sum.  The FP64 evaluation goes through world coordinates, at most ~40
+// roundings of terms that |R_w| |R_v|^T (|X| + |t_v|) + |t_w| bounds: 1e-14 of that is added.
+struct VgDir {
+  float M[9], t[3];
+  float Ca, Cb, m;
+};
+
+// Projects (X0, X1, z) with |Y_r| errors below E: q = Y_0,1 / Y_2 and the bound eq on its error.
+// Returns 1 in front (q, eq valid), 0 behind for certain, -1 not decided.  For e = E / Y2 <= 1/64,
+// |q - q*| <= e (1 + |q|) / (1 - e) plus 4u |q| for the reciprocal and the product.
+__device__ __forceinline__ int project(const VgDir& d, float X0, float X1, float z, float E, float& qu, float& qv,
+                                       float& eu, float& ev) {
+  constexpr float u = epo::kU32;
+  const float Y0 = fmaf(d.M[2], z, fmaf(d.M[1], X1, fmaf(d.M[0], X0, d.t[0])));
+  const float Y1 = fmaf(d.M[5], z, fmaf(d.M[4], X1, fmaf(d.M[3], X0, d.t[1])));
+  const float Y2 = fmaf(d.M[8], z, fmaf(d.M[7], X1, fmaf(d.M[6], X0, d.t[2])));
+  if (!(fabsf(Y2) > 1e-20f)) return -1;  // not a number, or where E could underflow
+  if (Y2 < -E) return 0;
+  float iz;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(iz) : "f"(Y2));
+  const float e = E * iz;
+  if (!(e >= 0.f && e <= 1.f / 64.f)) return -1;  // near the camera plane, or not a number
+  qu = Y0 * iz;
+  qv = Y1 * iz;
+  eu = fmaf(1.05f * e, 1.f + fabsf(qu), 4.f * u * fabsf(qu));
+  ev = fmaf(1.05f * e, 1.f + fabsf(qv), 4.f * u * fabsf(qv));
+  return 1;
+}
+
+// Pixel coordinate f q + c and its error bound (the rounded f and c, the FMA, the comparisons).
+__device__ __forceinline__ float pixel(float f, float c, float q, float eq, float& t) {
+  const float p = fmaf(f, q, c);
+  t = fmaf(f, eq, 6.f * epo::kU32 * (fabsf(p) + 2.f * fabsf(c)));
+  return p;
+}
+
+__global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views, const float* depth, int n, int stride,
+                                                          double tau, int per_block, uint2* counts) {
+  constexpr float u = epo::kU32;
+  __shared__ VgView vi, vj;
+  __shared__ VgDir fwd, bwd;
+  __shared__ double s_M[9];
+  __shared__ float s_n[2][8];  // per view: largest row and column sum of |R|, |t|, G
+  __shared__ int s_list[kVgExact];
+  __shared__ int s_count;
+  const int i = blockIdx.x / (n - 1), j0 = blockIdx.x % (n - 1), j = j0 + (j0 >= i);
+  {
+    constexpr int words = sizeof(VgView) / 8;
+    const double* a = reinterpret_cast<const double*>(views + i);
+    const double* b = reinterpret_cast<const double*>(views + j);
+    if (threadIdx.x < words) reinterpret_cast<double*>(&vi)[threadIdx.x] = a[threadIdx.x];
+    else if (threadIdx.x < 2 * words) reinterpret_cast<double*>(&vj)[threadIdx.x - words] = b[threadIdx.x - words];
+    if (threadIdx.x == 0) s_count = 0;
   }
-  const VgView vi = views[i], vj = views[j];
-  const int gw = (vi.W + stride - 1) / stride, gh = (vi.H + stride - 1) / stride;
-  unsigned valid = 0u, good = 0u;
-  for (int g = threadIdx.x; g < gw * gh; g += blockDim.x) {
-    const int x = (g % gw) * stride, y = (g / gw) * stride;
-    const double z = (double)depth[vi.off + (int64_t)y * vi.W + x];
-    if (!(z > 0.0) || !isfinite(z)) continue;
-    ++valid;
-    double xj, yj;
-    if (!reproject(vi, vj, (double)x, (double)y, z, xj, yj)) continue;
-    if (!(xj >= 0.0 && xj <= (double)(vj.W - 1) && yj >= 0.0 && yj <= (double)(vj.H - 1))) continue;
-    const int xn = (int)floor(add(xj, 0.5)), yn = (int)floor(add(yj, 0.5));  // nearest pixel
-    if (xn < 0 || xn >= vj.W || yn < 0 || yn >= vj.H) continue;
-    const double zj = (double)depth[vj.off + (int64_t)yn * vj.W + xn];
-    if (!(zj > 0.0) || !isfinite(zj)) continue;
-    double xb, yb;
-    if (!reproject(vj, vi, xj, yj, zj, xb, yb)) continue;
-    const double dx = sub(xb, (double)x), dy = sub(yb, (double)y);
-    if (__dsqrt_rn(add(mul(dx, dx), mul(dy, dy))) < tau) ++good;
-  }
-  // block sums in a fixed order
-  __shared__ unsigned s_v[kVgThreads], s_g[kVgThreads];
-  s_v[threadIdx.x] = valid;
-  s_g[threadIdx.x] = good;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      s_v[threadIdx.x] += s_v[threadIdx.x + w];
-      s_g[threadIdx.x] += s_g[threadIdx.x + w];
+  if (threadIdx.x < 9) {  // M = R_j R_i^T
+    const int r = threadIdx.x / 3, c = threadIdx.x % 3;
+    const double m = vj.T[4 * r] * vi.T[4 * c] + vj.T[4 * r + 1] * vi.T[4 * c + 1] + vj.T[4 * r + 2] * vi.T[4 * c + 2];
+    s_M[threadIdx.x] = m;
+    fwd.M[threadIdx.x] = (float)m;
+    bwd.M[3 * c + r] = (float)m;
+  } else if (threadIdx.x == 32 || threadIdx.x == 64) {
+    const int w = threadIdx.x / 32 - 1;
+    const VgView& v = w ? vj : vi;
+    float row = 0.f, col = 0.f, tm = 0.f;
+    for (int r = 0; r < 3; ++r) {
+      row = fmaxf(row, fabsf((float)v.T[4 * r]) + fabsf((float)v.T[4 * r + 1]) + fabsf((float)v.T[4 * r + 2]));
+      col = fmaxf(col, fabsf((float)v.T[r]) + fabsf((float)v.T[4 + r]) + fabsf((float)v.T[8 + r]));
+      tm = fmaxf(tm, fabsf((float)v.T[4 * r + 3]));
     }
-    __syncthreads();
+    const float gx = ((float)v.W + fabsf((float)v.K[2])) / (float)v.K[0];
+    const float gy = ((float)v.H + fabsf((float)v.K[3])) / (float)v.K[1];
+    s_n[w][0] = row;
+    s_n[w][1] = col;
+    s_n[w][2] = tm;
+    // images whose pixel coordinates are not exact in FP32 take no decision there
+    s_n[w][3] = v.W <= (1 << 22) && v.H <= (1 << 22) ? fmaxf(1.f, fmaxf(gx, gy)) : INFINITY;
   }
-  if (threadIdx.x == 0) frac[blockIdx.x] = s_v[0] > 0 ? (double)s_g[0] / (double)s_v[0] : 0.0;
+  __syncthreads();
+  if (threadIdx.x < 2) {  // t_ji = t_j - M t_i, and back t_ij = t_i - M^T t_j
+    const int w = threadIdx.x;
+    VgDir& d = w ? bwd : fwd;
+    const VgView& from = w ? vj : vi;
+    const VgView& to = w ? vi : vj;
+    const float* nf = s_n[w];
+    const float* nt = s_n[1 - w];
+    float m = 0.f, tm = 0.f;
+    for (int r = 0; r < 3; ++r) {
+      double t = to.T[4 * r + 3];
+      for (int c = 0; c < 3; ++c) t -= (w ? s_M[3 * c + r] : s_M[3 * r + c]) * from.T[4 * c + 3];
+      d.t[r] = (float)t;
+      tm = fmaxf(tm, fabsf((float)t));
+      m = fmaxf(m, fabsf(d.M[3 * r]) + fabsf(d.M[3 * r + 1]) + fabsf(d.M[3 * r + 2]));
+    }
+    const float mm = 1e-14f * nt[0] * nf[1];  // rows of |R_to| times columns of |R_from|
+    d.m = 1.01f * m;
+    d.Ca = 1.01f * nf[3] * (10.f * u * m + mm);
+    d.Cb = 1.01f * (10.f * u * tm + mm * nf[2] + 1e-14f * nt[2]);
+  }
+  __syncthreads();
+  const int gw = (vi.W + stride - 1) / stride, gh = (vi.H + stride - 1) / stride;
+  const int g0 = blockIdx.y * per_block, g1 = min(gw * gh, g0 + per_block);
+  const float fxi = (float)vi.K[0], fyi = (float)vi.K[1], cxi = (float)vi.K[2], cyi = (float)vi.K[3];
+  const float fxj = (float)vj.K[0], fyj = (float)vj.K[1], cxj = (float)vj.K[2], cyj = (float)vj.K[3];
+  const float rfx = (float)(1.0 / vi.K[0]), rfy = (float)(1.0 / vi.K[1]);
+  const float Wm1 = (float)(vj.W - 1), Hm1 = (float)(vj.H - 1), tf = (float)tau;
+  const float* di = depth + vi.off;
+  const float* dj = depth + vj.off;
+  unsigned valid = 0u, good = 0u;
+  const int dr = kVgThreads / gw, dc = kVgThreads % gw;
+  int row = (g0 + (int)threadIdx.x) / gw, col = (g0 + (int)threadIdx.x) % gw;
+  for (int g = g0 + threadIdx.x; g < g1; g += kVgThreads) {
+    const int x = col * stride, y = row * stride;
+    row += dr;
+    col += dc;
+    if (col >= gw) {
+      col -= gw;
+      ++row;
+    }
+    const float z = di[(int64_t)y * vi.W + x];
+    if (!(z > 0.f) || !isfinite(z)) continue;
+    ++valid;
+    int known = -1;  // 1 counted, 0 not, -1 an FP32 decision is in doubt
+    do {
+      const float xf = (float)x, yf = (float)y;
+      float qu, qv, eu, ev;
+      known = project(fwd, (xf - cxi) * rfx * z, (yf - cyi) * rfy * z, z, fmaf(z, fwd.Ca, fwd.Cb), qu, qv, eu, ev);
+      if (known != 1) break;
+      known = -1;
+      float tu, tv;
+      const float up = pixel(fxj, cxj, qu, eu, tu), vp = pixel(fyj, cyj, qv, ev, tv);
+      if (up < -tu || up - Wm1 > tu || vp < -tv || vp - Hm1 > tv) {
+        known = 0;  // outside view j
+        break;
+      }
+      const float fu = floorf(up), fv = floorf(vp), ru = up - fu, rv = vp - fv;
+      if (!(up >= tu && Wm1 - up >= tu && vp >= tv && Hm1 - vp >= tv && fabsf(ru - 0.5f) > tu && fabsf(rv - 0.5f) > tv)) break;
+      const int xn = (int)fu + (ru > 0.5f), yn = (int)fv + (rv > 0.5f);
+      const float zj = dj[(int64_t)yn * vj.W + xn];
+      if (!(zj > 0.f) || !isfinite(zj)) {
+        known = 0;
+        break;
+      }
+      const float E = fmaf(zj, fmaf(bwd.m, fmaxf(eu, ev), bwd.Ca), bwd.Cb);
+      float bu, bv;
+      known = project(bwd, qu * zj, qv * zj, zj, E, bu, bv, eu, ev);
+      if (known != 1) break;
+      known = -1;
+      const float dx = pixel(fxi, cxi, bu, eu, tu) - xf, dy = pixel(fyi, cyi, bv, ev, tv) - yf;
+      const float d = sqrtf(fmaf(dx, dx, dy * dy));
+      const float td = tu + tv + 8.f * u * (d + tf);
+      if (d + td < tf) known = 1;
+      else if (d - td > tf) known = 0;
+    } while (false);
+    good += known == 1;
+    if (known < 0) {
+      const int at = atomicAdd(&s_count, 1);
+      if (at < kVgExact) s_list[at] = g;
+      else good += trip_exact(vi, vj, depth, x, y, z, tau);
+    }
+  }
+  __syncthreads();
+  const int kept = min(s_count, kVgExact);
+  for (int k = threadIdx.x; k < kept; k += kVgThreads) {
+    const int x = s_list[k] % gw * stride, y = s_list[k] / gw * stride;
+    good += trip_exact(vi, vj, depth, x, y, di[(int64_t)y * vi.W + x], tau);
+  }
+  valid = __reduce_add_sync(0xffffffffu, valid);
+  good = __reduce_add_sync(0xffffffffu, good);
+  if ((threadIdx.x & 31) == 0) {
+    uint2* c = counts + (size_t)i * n + j;
+    if (valid) atomicAdd(&c->x, valid);
+    if (good) atomicAdd(&c->y, good);
+  }
 }
 
 }  // namespace
@@ -118,25 +279,42 @@ extern "C" epo_status epo_build_viewgraph(int32_t n_views, const int32_t* W, con
     if (!(hv[v].K[0] > 0) || !(hv[v].K[1] > 0)) return EPO_ERR_INVALID_ARG;
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  VgView* d_views = nullptr;
-  double* d_frac = nullptr;
-  std::vector<double> f((size_t)n * n);
+  // the view table and the pairs' counts in one allocation
+  const size_t view_bytes = sizeof(VgView) * n, count_bytes = sizeof(uint2) * (size_t)n * n;
+  static_assert(sizeof(VgView) % 8 == 0, "the counts follow the view table");
+  char* d_buf = nullptr;
+  std::vector<uint2> counts((size_t)n * n);
   epo_status rc = EPO_OK;
-  if (cudaMalloc(&d_views, sizeof(VgView) * n) != cudaSuccess ||
-      cudaMalloc(&d_frac, sizeof(double) * (size_t)n * n) != cudaSuccess) {
+  if (cudaMalloc(&d_buf, view_bytes + count_bytes) != cudaSuccess) {
     rc = EPO_ERR_OOM;
-  } else if (cudaMemcpyAsync(d_views, hv.data(), sizeof(VgView) * n, cudaMemcpyHostToDevice, st) != cudaSuccess) {
-    rc = EPO_ERR_CUDA;
   } else {
-    k_viewgraph<<<n * n, kVgThreads, 0, st>>>(d_views, depth_dev, n, stride, tau, d_frac);
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpyAsync(f.data(), d_frac, sizeof(double) * (size_t)n * n, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
+    const VgView* d_views = reinterpret_cast<const VgView*>(d_buf);
+    uint2* d_counts = reinterpret_cast<uint2*>(d_buf + view_bytes);
+    // one block per ordered pair; with few pairs each pair's grid is split over several blocks
+    // (at least 512 pixels each) so that they fill the GPU
+    int64_t grid = 1;
+    for (int v = 0; v < n; ++v)
+      grid = std::max(grid, (int64_t)((W[v] + stride - 1) / stride) * ((H[v] + stride - 1) / stride));
+    const int64_t pairs_n = (int64_t)n * (n - 1);
+    const int64_t split = std::min<int64_t>(std::max<int64_t>(1, kVgBlocks / std::max<int64_t>(pairs_n, 1)), (grid + 511) / 512);
+    const int per_block = (int)((grid + split - 1) / split);
+    if (cudaMemcpyAsync(d_buf, hv.data(), view_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemsetAsync(d_counts, 0, count_bytes, st) != cudaSuccess)
+      rc = EPO_ERR_CUDA;
+    if (rc == EPO_OK && pairs_n > 0) {
+      k_viewgraph<<<dim3((unsigned)pairs_n, (unsigned)split), kVgThreads, 0, st>>>(d_views, depth_dev, n, stride, tau,
+                                                                                  per_block, d_counts);
+      if (cudaGetLastError() != cudaSuccess) rc = EPO_ERR_CUDA;
+    }
+    if (rc == EPO_OK &&
+        (cudaMemcpyAsync(counts.data(), d_counts, count_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+         cudaStreamSynchronize(st) != cudaSuccess))
       rc = EPO_ERR_CUDA;
   }
-  if (d_views) cudaFree(d_views);
-  if (d_frac) cudaFree(d_frac);
+  if (d_buf) cudaFree(d_buf);
   if (rc != EPO_OK) return rc;
+  std::vector<double> f((size_t)n * n);
+  for (size_t k = 0; k < f.size(); ++k) f[k] = counts[k].x ? (double)counts[k].y / (double)counts[k].x : 0.0;
   // pairs kept in both directions, row-major
   int32_t m = 0;
   for (int i = 0; i < n; ++i)

@@ -34,3 +34,44 @@ def test_viewgraph_argument_checks():
     d = torch.zeros(16, device="cuda")
     with pytest.raises(epo.EpoError):
         epo.build_viewgraph([4], [4], [[0.0, 1.0, 1.5, 1.5]], np.eye(4)[:3].reshape(1, 12), d)
+
+
+@pytest.mark.parametrize("n,W,H,stride,tau,kind", [
+    (2, 61, 47, 1, 3.0, "smooth"), (3, 40, 30, 2, 0.75, "identical"), (5, 97, 33, 3, 1.5, "half"),
+    (9, 64, 48, 1, 3.0, "holes"), (4, 200, 150, 5, 10.0, "far"), (6, 80, 60, 2, 3.0, "sheared"),
+    (40, 24, 20, 1, 2.0, "smooth"), (4, 50, 40, 1, 3.0, "tiny"), (1, 8, 8, 1, 3.0, "smooth")])
+def test_viewgraph_counts_are_exact_where_decisions_are_close(n, W, H, stride, tau, kind):
+    """Scenes that put decisions of the round trip on their thresholds: identical views (every pixel
+    returns to itself, borders exactly on the border), shifts by half a pixel (every nearest-pixel
+    choice a tie), missing depths, poses far from the origin, matrices that are no rotations, depths
+    near the smallest floats."""
+    r = np.random.default_rng([n, W, H])
+    K = np.tile([1.1 * W, 1.1 * W, (W - 1) / 2, (H - 1) / 2], (n, 1))
+    y, x = np.mgrid[:H, :W]
+    depths = [(4 + np.sin(x / 9 + a) + 0.5 * np.cos(y / 7 + b)).astype(np.float32) for a, b in r.uniform(0, 6, (n, 2))]
+    T = np.zeros((n, 3, 4))
+    for v in range(n):
+        w = r.normal(0, 0.03, 3)
+        S = np.array([[0, -w[2], w[1]], [w[2], 0, -w[0]], [-w[1], w[0], 0]])
+        T[v, :, :3] = np.linalg.inv(np.eye(3) - S / 2) @ (np.eye(3) + S / 2)
+        T[v, :, 3] = r.normal(0, 0.2, 3)
+    if kind in ("identical", "half", "tiny"):
+        T[:] = np.eye(3, 4)
+        depths = [np.full((H, W), 4.0, np.float32)] * n
+    if kind == "half":
+        T[:, 0, 3] = np.arange(n) * 0.5 * 4.0 / K[0, 0]
+    if kind == "tiny":
+        depths = [(d * np.float32(10.0) ** r.integers(-44, -36, (H, W)).astype(np.float32)) for d in depths]
+    if kind == "holes":
+        for d in depths:
+            d[r.random((H, W)) < 0.3] = r.choice([0.0, -1.0, np.nan, np.inf])
+    if kind == "far":
+        T[:, :, 3] -= np.einsum("nij,j->ni", T[:, :, :3], [3e4, -2e4, 1e4])
+        K[:, 2:] += r.uniform(-40, 40, (n, 2))
+    if kind == "sheared":
+        T[:, :, :3] = T[:, :, :3] @ (np.eye(3) + r.normal(0, 0.05, (n, 3, 3)))
+    frac, pairs = epo.build_viewgraph(np.full(n, W), np.full(n, H), K, T.reshape(n, 12),
+                                      [torch.from_numpy(d).cuda() for d in depths], stride=stride, tau=tau, min_frac=0.125)
+    want = oracle.viewgraph(np.full(n, W), np.full(n, H), K, T.reshape(n, 12), depths, stride=stride, tau=tau)
+    assert np.array_equal(frac, want)
+    assert np.array_equal(pairs, oracle.viewgraph_pairs(want, 0.125))
