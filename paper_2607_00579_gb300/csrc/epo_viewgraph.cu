@@ -11,7 +11,7 @@
 // that evaluation is ~200 instructions of the 1/64-rate FP64 pipe per grid pixel (24 views of
 // 518x392 at stride 4: 2.5 ms), so every grid pixel first runs in FP32 beside a bound on its error,
 // and only those with a decision inside the bound (well under 1 % of them) are kept in shared
-// memory and evaluated in FP64, 32 to a warp (the same 24 views: 2544 -> 205 us for the whole call).
+// memory and evaluated in FP64, 32 to a warp (the same 24 views: 2544 -> 166 us for the whole call).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -71,7 +71,8 @@ __device__ __noinline__ bool trip_exact(const VgView& vi, const VgView& vj, cons
 }
 
 constexpr int kVgThreads = 256;
-constexpr int kVgExact = 1024;   // grid pixels a block keeps for the FP64 evaluation
+constexpr int kVgRound = 1024;           // grid pixels between two looks at the kept ones
+constexpr int kVgExact = 2 * kVgRound;   // room for the kept ones: evaluated once half full
 constexpr int kVgBlocks = 8 * 152;  // one wave of resident blocks: fewer pairs are split over several
 
 // One direction of a pair in FP32: Y = M X + t, and the constants of the bound
@@ -115,7 +116,8 @@ __device__ __forceinline__ float pixel(float f, float c, float q, float eq, floa
   return p;
 }
 
-__global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views, const float* depth, int n, int stride,
+// Five blocks per SM (48 registers): 166 us for the call on 24 views; three 177, four 169, six 195.
+__global__ void __launch_bounds__(kVgThreads, 5) k_viewgraph(const VgView* views, const float* depth, int n, int stride,
                                                           double tau, int per_block, uint2* counts) {
   constexpr float u = epo::kU32;
   __shared__ VgView vi, vj;
@@ -154,8 +156,9 @@ __global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views
     s_n[w][0] = row;
     s_n[w][1] = col;
     s_n[w][2] = tm;
-    // images whose pixel coordinates are not exact in FP32 take no decision there
-    s_n[w][3] = v.W <= (1 << 22) && v.H <= (1 << 22) ? fmaxf(1.f, fmaxf(gx, gy)) : INFINITY;
+    // images whose pixel coordinates are not exact in FP32, or whose pixels an int does not number,
+    // take no decision there
+    s_n[w][3] = v.W <= (1 << 22) && v.H <= (1 << 22) && (int64_t)v.W * v.H <= INT32_MAX ? fmaxf(1.f, fmaxf(gx, gy)) : INFINITY;
   }
   __syncthreads();
   if (threadIdx.x < 2) {  // t_ji = t_j - M t_i, and back t_ij = t_i - M^T t_j
@@ -188,63 +191,92 @@ __global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views
   const float* di = depth + vi.off;
   const float* dj = depth + vj.off;
   unsigned valid = 0u, good = 0u;
-  const int dr = kVgThreads / gw, dc = kVgThreads % gw;
-  int row = (g0 + (int)threadIdx.x) / gw, col = (g0 + (int)threadIdx.x) % gw;
-  for (int g = g0 + threadIdx.x; g < g1; g += kVgThreads) {
-    const int x = col * stride, y = row * stride;
-    row += dr;
-    col += dc;
-    if (col >= gw) {
-      col -= gw;
-      ++row;
-    }
-    const float z = di[(int64_t)y * vi.W + x];
-    if (!(z > 0.f) || !isfinite(z)) continue;
-    ++valid;
-    int known = -1;  // 1 counted, 0 not, -1 an FP32 decision is in doubt
-    do {
-      const float xf = (float)x, yf = (float)y;
-      float qu, qv, eu, ev;
-      known = project(fwd, (xf - cxi) * rfx * z, (yf - cyi) * rfy * z, z, fmaf(z, fwd.Ca, fwd.Cb), qu, qv, eu, ev);
-      if (known != 1) break;
-      known = -1;
-      float tu, tv;
-      const float up = pixel(fxj, cxj, qu, eu, tu), vp = pixel(fyj, cyj, qv, ev, tv);
-      if (up < -tu || up - Wm1 > tu || vp < -tv || vp - Hm1 > tv) {
-        known = 0;  // outside view j
-        break;
-      }
-      const float fu = floorf(up), fv = floorf(vp), ru = up - fu, rv = vp - fv;
-      if (!(up >= tu && Wm1 - up >= tu && vp >= tv && Hm1 - vp >= tv && fabsf(ru - 0.5f) > tu && fabsf(rv - 0.5f) > tv)) break;
-      const int xn = (int)fu + (ru > 0.5f), yn = (int)fv + (rv > 0.5f);
-      const float zj = dj[(int64_t)yn * vj.W + xn];
-      if (!(zj > 0.f) || !isfinite(zj)) {
-        known = 0;
-        break;
-      }
-      const float E = fmaf(zj, fmaf(bwd.m, fmaxf(eu, ev), bwd.Ca), bwd.Cb);
-      float bu, bv;
-      known = project(bwd, qu * zj, qv * zj, zj, E, bu, bv, eu, ev);
-      if (known != 1) break;
-      known = -1;
-      const float dx = pixel(fxi, cxi, bu, eu, tu) - xf, dy = pixel(fyi, cyi, bv, ev, tv) - yf;
-      const float d = sqrtf(fmaf(dx, dx, dy * dy));
-      const float td = tu + tv + 8.f * u * (d + tf);
-      if (d + td < tf) known = 1;
-      else if (d - td > tf) known = 0;
-    } while (false);
-    good += known == 1;
-    if (known < 0) {
-      const int at = atomicAdd(&s_count, 1);
-      if (at < kVgExact) s_list[at] = g;
-      else good += trip_exact(vi, vj, depth, x, y, z, tau);
-    }
+  // two grid pixels per thread in flight: each trip is two dependent loads, and the kernel waits
+  // for them rather than for its arithmetic (one in flight: 205 us for the call on 24 views of
+  // 518x392, two: 166)
+  constexpr int ILP = 2;
+  constexpr int kStep = ILP * kVgThreads;
+  const int dr = kStep / gw, dc = kStep % gw;
+  int row[ILP], col[ILP];
+#pragma unroll
+  for (int k = 0; k < ILP; ++k) {
+    const int g = g0 + k * kVgThreads + (int)threadIdx.x;
+    row[k] = g / gw;
+    col[k] = g % gw;
   }
-  __syncthreads();
-  const int kept = min(s_count, kVgExact);
-  for (int k = threadIdx.x; k < kept; k += kVgThreads) {
-    const int x = s_list[k] % gw * stride, y = s_list[k] / gw * stride;
-    good += trip_exact(vi, vj, depth, x, y, di[(int64_t)y * vi.W + x], tau);
+  for (int round = g0; round < g1; round += kVgRound) {
+    const int end = min(g1, round + kVgRound);
+    for (int base = round; base < end; base += kStep) {
+      int known[ILP];  // 1 counted, 0 not, -1 an FP32 decision is in doubt, 2 not decided yet
+      float z[ILP], qu[ILP], qv[ILP], eu[ILP], ev[ILP], zj[ILP], xf[ILP], yf[ILP];
+      int at[ILP];
+#pragma unroll
+      for (int k = 0; k < ILP; ++k) {
+        const int x = col[k] * stride, y = row[k] * stride;
+        const bool in = base + k * kVgThreads + (int)threadIdx.x < end;
+        z[k] = in ? di[(int64_t)y * vi.W + x] : 0.f;
+        xf[k] = (float)x;
+        yf[k] = (float)y;
+        row[k] += dr;
+        col[k] += dc;
+        if (col[k] >= gw) {
+          col[k] -= gw;
+          ++row[k];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < ILP; ++k) {
+        known[k] = 0;
+        at[k] = -1;
+        if (!(z[k] > 0.f) || !isfinite(z[k])) continue;
+        ++valid;
+        known[k] = project(fwd, (xf[k] - cxi) * rfx * z[k], (yf[k] - cyi) * rfy * z[k], z[k], fmaf(z[k], fwd.Ca, fwd.Cb),
+                           qu[k], qv[k], eu[k], ev[k]);
+        if (known[k] != 1) continue;
+        float tu, tv;
+        const float up = pixel(fxj, cxj, qu[k], eu[k], tu), vp = pixel(fyj, cyj, qv[k], ev[k], tv);
+        known[k] = up < -tu || up - Wm1 > tu || vp < -tv || vp - Hm1 > tv ? 0 : -1;  // outside view j, or perhaps
+        const float fu = floorf(up), fv = floorf(vp), ru = up - fu, rv = vp - fv;
+        if (up >= tu && Wm1 - up >= tu && vp >= tv && Hm1 - vp >= tv && fabsf(ru - 0.5f) > tu && fabsf(rv - 0.5f) > tv) {
+          known[k] = 2;
+          at[k] = ((int)fv + (rv > 0.5f)) * vj.W + (int)fu + (ru > 0.5f);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < ILP; ++k) zj[k] = at[k] >= 0 ? dj[at[k]] : 0.f;
+#pragma unroll
+      for (int k = 0; k < ILP; ++k) {
+        if (known[k] == 2) {
+          known[k] = 0;
+          if (zj[k] > 0.f && isfinite(zj[k])) {
+            const float E = fmaf(zj[k], fmaf(bwd.m, fmaxf(eu[k], ev[k]), bwd.Ca), bwd.Cb);
+            float bu, bv;
+            known[k] = project(bwd, qu[k] * zj[k], qv[k] * zj[k], zj[k], E, bu, bv, eu[k], ev[k]);
+            if (known[k] == 1) {
+              float tu, tv;
+              const float dx = pixel(fxi, cxi, bu, eu[k], tu) - xf[k], dy = pixel(fyi, cyi, bv, ev[k], tv) - yf[k];
+              const float d = sqrtf(fmaf(dx, dx, dy * dy));
+              const float td = tu + tv + 8.f * u * (d + tf);
+              known[k] = d + td < tf ? 1 : (d - td > tf ? 0 : -1);
+            }
+          }
+        }
+        good += known[k] == 1;
+        if (known[k] < 0) s_list[atomicAdd(&s_count, 1)] = base + k * kVgThreads + (int)threadIdx.x;
+      }
+    }
+    __syncthreads();
+    const int kept = s_count;
+    __syncthreads();  // every thread has read it before the next round appends
+    if (kept > kVgExact - kVgRound || end == g1) {
+      for (int k = threadIdx.x; k < kept; k += kVgThreads) {
+        const int x = s_list[k] % gw * stride, y = s_list[k] / gw * stride;
+        good += trip_exact(vi, vj, depth, x, y, di[(int64_t)y * vi.W + x], tau);
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) s_count = 0;
+      __syncthreads();
+    }
   }
   valid = __reduce_add_sync(0xffffffffu, valid);
   good = __reduce_add_sync(0xffffffffu, good);
