@@ -116,16 +116,19 @@ typedef struct {
   int32_t autotune;          /* 1: pick the kernel schedule by timing on first use;
                                 2: the same, each timed launch starting from a cold L2 */
   int32_t gather;            /* EPO_GATHER_* (AUTO = TEX unless autotuned) */
-  int32_t block_threads;     /* 0 = default (256); else 64..512, multiple of 32 */
-  int32_t records_per_thread;/* 0 = default (2); 1, 2, 4 or 8 (two in flight at a time;
-                                refine scenes: 2) */
+  int32_t block_threads;     /* 0 = default (256, or 128 with four records per thread where that
+                                is faster and the rest of the schedule is the default too);
+                                else 64..512, multiple of 32 */
+  int32_t records_per_thread;/* 0 = default (2, or 4 as above); 1, 2, 4 or 8 (two in flight at a
+                                time; refine scenes: 2) */
   int32_t grid_blocks;       /* 0 = default (persistent: SMs x resident blocks) */
   int32_t timing;            /* 1: bracket the edge kernel with CUDA events (epo_kernel_time) */
   int32_t tail_pairs;        /* work items of the last wave (as many as the grid has blocks):
                                 0 = each covers all of its view's pairs, like the others;
                                 n > 0 = split into items of at most n pairs, so that the
                                 blocks finish together; -1 = default (autotuned when
-                                autotune is on, else 0); n <= -2 = every work item, not
+                                autotune is on, else chosen from the amount of work);
+                                n <= -2 = every work item, not
                                 only the last wave's, covers at most -n pairs */
   int32_t refine;            /* 1: the scene also carries the focal and depth refinement of
                                 Section 3 (Eq. 4: f_i = f_i^0 (1 + gamma_i) for both focal

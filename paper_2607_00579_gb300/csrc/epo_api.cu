@@ -51,6 +51,14 @@ float half_bits_to_float(uint16_t h) {
   return f;
 }
 
+// Schedule of the edge kernel.
+struct Sched {
+  int gather = GATHER_TEX, rpt = 2;
+  int halves = 1;  // 2: the block does the work item of one twice as wide (k_edge_pose, HALVES)
+  int block = 256;
+  int tail = 0;    // pairs per work item of the last wave (0 = not split)
+};
+
 }  // namespace
 
 struct epo_scene {
@@ -64,7 +72,7 @@ struct epo_scene {
   int64_t n_records = 0, n_dropped = 0, evals = 0;
   int sm_count = 0;
   // schedule
-  int gather = GATHER_TEX, block = 256, rpt = 4, grid = 0;
+  Sched sch;
   bool tuned = false;
   // host tables
   std::vector<ViewDev> views;
@@ -84,7 +92,6 @@ struct epo_scene {
   int tiles_for = -1;   // tile size the current table was built for
   int tiles_tail = -1;  // and its tail split
   int tiles_grid = -1;  // over the last wave of this many blocks
-  int tail = 0;         // pairs per work item of the last wave (0 = not split)
   struct TileTable {
     int tile, tail, grid;
     TileDev* p;
@@ -431,7 +438,7 @@ StepArgs step_args(epo_scene* S, const double* T_eval, const double* gscale) {
   return a;
 }
 
-int resident_blocks(epo_scene* S, int gather, int rpt, int block);
+int resident_blocks(epo_scene* S, const Sched& sc);
 
 // Work items of the edge kernel, in the order the blocks claim them: (view, records
 // [begin, begin + n), pairs [q0, q1) of the view's outgoing pair list).  Each item covers
@@ -493,13 +500,13 @@ epo_status build_tiles(epo_scene* S, int tile, int tail, int grid) {
 // Work items of a schedule: block * rpt records each; with tail > 0 the last wave is one item
 // per resident block (items of at most `tail` pairs), with tail < 0 every item covers at most
 // -tail pairs (more, smaller items).
-epo_status build_tiles(epo_scene* S, int gather, int rpt, int block, int tail) {
-  if (tail < 0) return build_tiles(S, block * rpt, -tail, INT_MAX);
-  return build_tiles(S, block * rpt, tail, tail ? resident_blocks(S, gather, rpt, block) : 0);
+epo_status build_tiles(epo_scene* S, const Sched& sc) {
+  if (sc.tail < 0) return build_tiles(S, sc.block * sc.rpt, -sc.tail, INT_MAX);
+  return build_tiles(S, sc.block * sc.rpt, sc.tail, sc.tail ? resident_blocks(S, sc) : 0);
 }
 
 // The work items of the current schedule.
-epo_status build_tiles(epo_scene* S) { return build_tiles(S, S->gather, S->rpt, S->block, S->tail); }
+epo_status build_tiles(epo_scene* S) { return build_tiles(S, S->sch); }
 
 EdgeArgs edge_args(epo_scene* S) {
   EdgeArgs a;
@@ -519,7 +526,6 @@ EdgeArgs edge_args(epo_scene* S) {
   a.q_count = S->d_qcount;
   a.q_overflow = S->d_qoverflow;
   a.tile_counter = S->d_tile_counter;
-  a.max_pairs = S->max_pairs;
   a.pair_active = S->d_active;
   a.tex = S->d_tex;
   a.pair_acc = S->d_pair_acc;
@@ -542,28 +548,93 @@ EdgeArgs edge_args(epo_scene* S) {
   return a;
 }
 
+// Most pairs of one work item: the rows of the kernel's per-pair sums in shared memory.
+int item_pairs(epo_scene* S, const Sched& sc) { return sc.tail < 0 ? std::min(S->max_pairs, -sc.tail) : S->max_pairs; }
+
 // Blocks of the persistent edge kernel: every SM holds as many as its registers, threads
 // and shared memory allow (or the caller's fixed grid size).
-int resident_blocks(epo_scene* S, int gather, int rpt, int block) {
+int resident_blocks(epo_scene* S, const Sched& sc) {
   if (S->opt.grid_blocks > 0) return S->opt.grid_blocks;
   int per_sm = 0;
-  const void* k = edge_kernel_ptr(MODE_FUSED, S->refine, S->rec_dtype, S->map_dtype, gather, rpt);
-  const size_t smem = edge_smem_bytes(rpt, block, S->max_pairs, S->refine);
+  const void* k = edge_kernel_ptr(MODE_FUSED, S->refine, S->rec_dtype, S->map_dtype, sc.gather, sc.rpt, sc.halves);
+  const size_t smem = edge_smem_bytes(sc.rpt, sc.block, item_pairs(S, sc), S->refine, sc.halves);
   if (smem > 48 * 1024 && k) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (!k || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem) != cudaSuccess || per_sm < 1)
-    per_sm = std::max(1, 1024 / block);
+  if (!k || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, sc.block, smem) != cudaSuccess || per_sm < 1)
+    per_sm = std::max(1, 1024 / sc.block);
   return std::max(1, S->sm_count * per_sm);
 }
 
 // Launch size of the edge kernel for the current tile table.
-int grid_for(epo_scene* S, int gather, int rpt, int block) {
-  return std::max(1, std::min(resident_blocks(S, gather, rpt, block), std::max(S->n_tiles, 1)));
+int grid_for(epo_scene* S, const Sched& sc) {
+  return std::max(1, std::min(resident_blocks(S, sc), std::max(S->n_tiles, 1)));
 }
 
 constexpr size_t kMaxSmem = 227 * 1024;
 
-bool schedule_fits(epo_scene* S, int rpt, int block) {
-  return (!S->refine || rpt == 2) && edge_smem_bytes(rpt, block, S->max_pairs, S->refine) <= kMaxSmem;
+bool schedule_fits(epo_scene* S, const Sched& sc) {
+  return (!S->refine || sc.rpt == 2) && edge_smem_bytes(sc.rpt, sc.block, item_pairs(S, sc), S->refine, sc.halves) <= kMaxSmem;
+}
+
+// The schedule of a pose-only scene whose options leave it to the library.  All of these give the
+// same bits: a work item is 512 records, either two per thread of 256 threads or four per thread of
+// 128 (two halves, k_edge_pose), and a split by pairs moves whole sums to other blocks.
+//
+// With U = work items x pairs (those a step evaluates) and G = 1368 resident 128-thread blocks:
+//  - U >= 4 G: 128 threads, items of about sqrt(U / 2G) pairs.  On a full SM a pair of one item
+//    takes ~3.6 us, so a block that claims a whole item last keeps the others waiting; each item
+//    costs about a quarter of a pair more.  U / G + U / (4 G n) + n / 2 is least there.  Once that
+//    nears the whole item nothing is split.
+//  - below, 256 threads: one wave of items if at most 4 pairs each make one (a block that runs alone
+//    is bound by the latency of its pairs, one after the other); else items of 4 where the whole ones
+//    fill the SMs or are longer than 8.
+// Step, microseconds, 256 threads unsplit -> this rule: 8 views of 128x96 all pairs 24.8 -> 18.6;
+// 14 of 319x241 35.3 -> 24.8; 32 of 256x192 29.6 -> 22.6; 30 of 518x392 with 12
+// pairs a view 39.1 -> 33.0; 16 of 518x392 30.5, not split (31.0 in fours); 120 of 256x192 46.7 ->
+// 37.3; 32 of 518x392 51.1 -> 49.2; 48 of 518x392 67.4 -> 65.6; 20 of 518x518 all pairs, BF16
+// 88.6 -> 75.0; 96 of 518x392 92.8 -> 82.7; 120 of 518x392 157 -> 147; 200 of 518x392 333 -> 311; 300 of
+// 518x518, BF16 652 -> 594; 24 uneven scenes 689 -> 625.
+void default_schedule(epo_scene* S) {
+  const Sched wide = S->sch;  // 256 threads, two records per thread
+  if (wide.block != 256 || wide.rpt != 2) return;
+  const double G = 1368.0;
+  double tiles = 0.0, U = 0.0;
+  for (int v = 0; v < S->n_views; ++v) {
+    const int k = S->src_pair_off[v + 1] - S->src_pair_off[v];
+    const double t = k ? (double)((S->views[v].n_rec + 511) / 512) : 0.0;
+    tiles += t;
+    U += t * k;
+  }
+  if (!(U > 0.0)) return;
+  double share = 1.0;  // of the pairs a step evaluates (Algorithm 3's budget)
+  if (S->opt.pair_budget > 0) {
+    double act = 0.0;
+    for (int sc = 0; sc < S->n_scenes; ++sc)
+      act += std::min(S->opt.pair_budget, S->scene_pair_off[sc + 1] - S->scene_pair_off[sc]);
+    share = act / S->n_pairs;
+  }
+  const double k = U / tiles;  // pairs per view
+  if (U * share >= 4.0 * G) {
+    S->sch.block = 128;
+    S->sch.rpt = 4;
+    S->sch.halves = 2;
+    const double n = std::max(1.0, floor(sqrt(U * share / (2.0 * G)) / share + 0.5));
+    const double even = ceil(k / ceil(k / n));  // pieces of equal size
+    if (n < 0.75 * k) S->sch.tail = -(int)even;
+    if (!schedule_fits(S, S->sch)) S->sch = wide;
+    return;
+  }
+  const double slots = S->sm_count * 4.0;
+  for (int n = 1; n <= 4 && n < S->max_pairs; ++n) {
+    double items = 0.0;
+    for (int v = 0; v < S->n_views; ++v) {
+      const int kv = S->src_pair_off[v + 1] - S->src_pair_off[v];
+      items += (double)((S->views[v].n_rec + 511) / 512) * ((kv + n - 1) / n);
+    }
+    if (items <= slots || (n == 4 && (k > 8.0 || tiles > 0.9 * slots))) {
+      S->sch.tail = -n;
+      return;
+    }
+  }
 }
 
 // Record stage event k on stream s (inside a capture it becomes an event-record node).
@@ -583,16 +654,17 @@ epo_status mark(epo_scene* S, int k, cudaStream_t s) {
     if (m_ != EPO_OK) return m_;           \
   } while (0)
 
-epo_status run_edge(epo_scene* S, int mode, int gather, int rpt, int block, int tail, cudaStream_t s) {
-  if (!schedule_fits(S, rpt, block))
+epo_status run_edge(epo_scene* S, int mode, const Sched& sc, cudaStream_t s) {
+  if (!schedule_fits(S, sc))
     return fail(S, EPO_ERR_INVALID_ARG, "schedule needs more shared memory than a block has");
-  if (gather == GATHER_MIX && (S->refine || rpt == 1))
+  if (sc.gather == GATHER_MIX && (S->refine || sc.rpt == 1))
     return fail(S, EPO_ERR_INVALID_ARG, "the mixed gather needs a pose-only scene and two or more records per thread");
-  epo_status st = build_tiles(S, gather, rpt, block, tail);
+  epo_status st = build_tiles(S, sc);
   if (st != EPO_OK) return st;
   EdgeArgs ea = edge_args(S);
-  int grid = grid_for(S, gather, rpt, block);
-  CK(launch_edge(ea, mode, S->refine, S->rec_dtype, S->map_dtype, gather, rpt, block, grid, s));
+  ea.max_pairs = item_pairs(S, sc);
+  int grid = grid_for(S, sc);
+  CK(launch_edge(ea, mode, S->refine, S->rec_dtype, S->map_dtype, sc.gather, sc.rpt, sc.halves, sc.block, grid, s));
   MARK(2, s);
   return EPO_OK;
 }
@@ -605,7 +677,7 @@ epo_status enqueue_loss_grad(epo_scene* S, cudaStream_t s, const double* T_eval)
   if (S->refine) CK(launch_refine_intrinsics(a, s));
   CK(launch_pair_setup(a, MODE_FUSED, s));
   MARK(1, s);
-  epo_status st = run_edge(S, MODE_FUSED, S->gather, S->rpt, S->block, S->tail, s);
+  epo_status st = run_edge(S, MODE_FUSED, S->sch, s);
   if (st != EPO_OK) return st;
   CK(launch_poses(a, 1, s));
   MARK(3, s);
@@ -627,7 +699,7 @@ epo_status enqueue_step(epo_scene* S, cudaStream_t s, double* host_out = nullptr
   if (S->refine) CK(launch_refine_intrinsics(a, s));
   CK(launch_pair_setup(a, MODE_FUSED, s));
   MARK(1, s);
-  epo_status st = run_edge(S, MODE_FUSED, S->gather, S->rpt, S->block, S->tail, s);
+  epo_status st = run_edge(S, MODE_FUSED, S->sch, s);
   if (st != EPO_OK) return st;
   CK(launch_poses(a, 2, s));
   if (S->pose_mlp) {  // the poses' gradient through phi and the MLP; AdamW (advances the step)
@@ -1205,17 +1277,20 @@ epo_status create_impl(int32_t n_scenes, const epo_scene_desc* descs, const epo_
     if (o.timing)
       for (auto& e2 : S->ev) CK(cudaEventCreate(&e2));
     // schedule
-    S->block = o.block_threads ? o.block_threads : 256;
-    S->rpt = o.records_per_thread ? o.records_per_thread : 2;
+    S->sch.block = o.block_threads ? o.block_threads : 256;
+    S->sch.rpt = o.records_per_thread ? o.records_per_thread : 2;
     // AUTO is the texture gather: one instruction and one address per footprint instead of four
     // loads, the same values, and never slower over the scenes measured at the default 256 threads
     // and two records per thread (edge stage, plain loads -> texture): 8 views of 128x96 18.0 ->
     // 18.4 us, 14 of 319x241 26.2 -> 26.1, 32 of 518x392 57.6 -> 42.9, 48 of 518x392 75.7 -> 53.3,
     // 96 of 518x518 in BF16 225 -> 168, a 24-scene batch 856 -> 660, 32 views with refinement
     // 55.3 -> 51.2
-    S->gather = o.gather == EPO_GATHER_LDG ? GATHER_LDG : (o.gather == EPO_GATHER_MIX ? GATHER_MIX : GATHER_TEX);
-    if (!schedule_fits(S, S->rpt, S->block)) S->block = 128;
-    S->tail = o.tail_pairs == -1 ? 0 : o.tail_pairs;
+    S->sch.gather = o.gather == EPO_GATHER_LDG ? GATHER_LDG : (o.gather == EPO_GATHER_MIX ? GATHER_MIX : GATHER_TEX);
+    if (!schedule_fits(S, S->sch)) S->sch.block = 128;
+    S->sch.tail = o.tail_pairs == -1 ? 0 : o.tail_pairs;
+    if (!S->refine && S->sch.gather == GATHER_TEX && o.block_threads == 0 && o.records_per_thread == 0 &&
+        o.grid_blocks == 0 && o.tail_pairs == -1)
+      default_schedule(S);
     epo_status bs = build_tiles(S);
     if (bs != EPO_OK) return bs;
     CK(cudaStreamSynchronize(st));
@@ -1339,12 +1414,12 @@ epo_status epo_scene_info_get(epo_scene_t S, epo_scene_info* info) {
   info->record_bytes = S->n_records * (S->rec_dtype ? 8 : 16);
   info->map_bytes = S->map_elems * (S->map_dtype ? 2 : 4);
   info->n_tiles = S->n_tiles;
-  info->gather = S->gather;
-  info->block_threads = S->block;
-  info->records_per_thread = S->rpt;
-  info->grid_blocks = grid_for(S, S->gather, S->rpt, S->block);
+  info->gather = S->sch.gather;
+  info->block_threads = S->sch.block;
+  info->records_per_thread = S->sch.rpt;
+  info->grid_blocks = grid_for(S, S->sch);
   info->kernels_per_step = 3 + S->refine + S->subsample + S->opt.schedule + S->depth_opt + 3 * S->pose_mlp;
-  info->tail_pairs = S->tail;
+  info->tail_pairs = S->sch.tail;
   return EPO_OK;
 }
 
@@ -1546,7 +1621,7 @@ epo_status epo_forward_dev(epo_scene_t S, const double* xi_dev, double* loss_dev
   if (S->refine) CK(launch_refine_intrinsics(a, S->stream));
   CK(launch_pair_setup(a, MODE_FWD, S->stream));
   MARK(1, S->stream);
-  st = run_edge(S, MODE_FWD, S->gather, S->rpt, S->block, S->tail, S->stream);
+  st = run_edge(S, MODE_FWD, S->sch, S->stream);
   if (st != EPO_OK) return st;
   CK(launch_poses(a, 0, S->stream));
   MARK(3, S->stream);
@@ -1565,7 +1640,7 @@ epo_status epo_backward_dev(epo_scene_t S, const double* xi_dev, const double* d
   if (S->refine) CK(launch_refine_intrinsics(a, S->stream));
   CK(launch_pair_setup(a, MODE_BWD, S->stream));
   MARK(1, S->stream);
-  epo_status st = run_edge(S, MODE_BWD, S->gather, S->rpt, S->block, S->tail, S->stream);
+  epo_status st = run_edge(S, MODE_BWD, S->sch, S->stream);
   if (st != EPO_OK) return st;
   CK(launch_poses(a, 1, S->stream));
   MARK(3, S->stream);
@@ -1756,7 +1831,7 @@ epo_status epo_refine_loss_and_grad(epo_scene_t S, double* loss, double* grad, d
   if (S->subsample) CK(launch_subsample(a, s));
   CK(launch_refine_intrinsics(a, s));
   CK(launch_pair_setup(a, MODE_FUSED, s));
-  st = run_edge(S, MODE_FUSED, S->gather, S->rpt, S->block, S->tail, s);
+  st = run_edge(S, MODE_FUSED, S->sch, s);
   if (st != EPO_OK) return st;
   CK(launch_poses(a, 1, s));
   CK(launch_depth(a, 0, s));
@@ -1832,7 +1907,7 @@ epo_status epo_autotune(epo_scene_t S) {
   if (!S) return fail(S, EPO_ERR_INVALID_ARG, "null scene");
   S->tuned = true;  // also guards against recursion through maybe_autotune
   struct Cand {
-    int g, r, b, t;
+    Sched sc;
     std::vector<float> ms;
     float med;
   };
@@ -1845,8 +1920,9 @@ epo_status epo_autotune(epo_scene_t S) {
         if (S->opt.gather == EPO_GATHER_TEX && g != GATHER_TEX) continue;
         if (S->opt.gather == EPO_GATHER_MIX && g != GATHER_MIX) continue;
         if (g == GATHER_MIX && (S->refine || r == 1)) continue;
-        if (!schedule_fits(S, r, b)) continue;
-        cands.push_back({g, r, b, tail0, {}, 0.f});
+        const Sched sc{g, r, 1, b, tail0};
+        if (!schedule_fits(S, sc)) continue;
+        cands.push_back({sc, {}, 0.f});
       }
   if (cands.empty()) return fail(S, EPO_ERR_INVALID_ARG, "no edge-kernel schedule fits this scene");
   cudaEvent_t e0, e1;
@@ -1867,7 +1943,7 @@ epo_status epo_autotune(epo_scene_t S) {
   int fill = 0;
   // one launch of candidate c; its time is appended when `timed`
   auto launch = [&](Cand& c, bool timed) -> epo_status {
-    epo_status st = build_tiles(S, c.g, c.r, c.b, c.t);  // outside the timed interval
+    epo_status st = build_tiles(S, c.sc);  // outside the timed interval
     if (st != EPO_OK) return st;
     if (flush) {
       CK(cudaMemsetAsync(flush, ++fill & 0xff, flush_bytes, S->stream));
@@ -1878,7 +1954,7 @@ epo_status epo_autotune(epo_scene_t S) {
     if (S->refine) CK(launch_refine_intrinsics(a, S->stream));
     CK(launch_pair_setup(a, MODE_FUSED, S->stream));
     CK(cudaEventRecord(e0, S->stream));
-    st = run_edge(S, MODE_FUSED, c.g, c.r, c.b, c.t, S->stream);
+    st = run_edge(S, MODE_FUSED, c.sc, S->stream);
     if (st != EPO_OK) return st;
     CK(cudaEventRecord(e1, S->stream));
     CK(cudaEventSynchronize(e1));
@@ -1907,7 +1983,7 @@ epo_status epo_autotune(epo_scene_t S) {
       for (size_t k = 0; k < n4; ++k)
         for (int t : {2, 1}) {
           Cand c = cands[k];
-          c.t = t;
+          c.sc.tail = t;
           c.ms.clear();
           cands.push_back(c);
         }
@@ -1929,10 +2005,7 @@ epo_status epo_autotune(epo_scene_t S) {
     c.med = median(c.ms);
     if (c.med < best->med) best = &c;
   }
-  S->gather = best->g;
-  S->rpt = best->r;
-  S->block = best->b;
-  S->tail = best->t;
+  S->sch = best->sc;
   S->graph_dirty = true;
   return build_tiles(S);
 }

@@ -603,11 +603,18 @@ struct AmbRef {
 constexpr int kAmbCapPose = EPO_POSE_AMBCAP;
 constexpr int kAmbRunPose = kAmbCapPose * 3 / 8;
 
-template <int MODE, int REC, int MAP, int GATHER, int RPT>
+// HALVES = 2 (four records per thread): the block does the work item of one twice as wide with two
+// records per thread, in the same order.  Thread t is its threads t and t + blockDim in turn: the
+// records t, t + 2 blockDim of one half, then t + blockDim, t + 3 blockDim of the other, each half
+// with its own sums, warp reductions and shared-memory rows, so every sum is formed exactly as there.
+// The pair's constants are read once for four records instead of two, and nine such blocks are
+// resident per SM where four of the wide ones are.
+template <int MODE, int REC, int MAP, int GATHER, int RPT, int HALVES = 1>
 __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
+  static_assert(HALVES == 1 || (HALVES == 2 && RPT == 4), "two halves of two records");
   extern __shared__ float4 s_dyn[];
   float4* s_X = s_dyn;                                                    // [blockDim * RPT]
-  float* s_part = reinterpret_cast<float*>(s_X + blockDim.x * RPT);      // [warps][max_pairs][kAcc]
+  float* s_part = reinterpret_cast<float*>(s_X + blockDim.x * RPT);      // [HALVES * warps][max_pairs][kAcc]
   __shared__ int s_tile, s_next;
   __shared__ int s_amb_n;
   __shared__ AmbRef s_amb[kAmbCapPose];
@@ -659,17 +666,19 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
                   r7 = P.r[7], r8 = P.r[8], t0 = P.t[0], t1 = P.t[1], t2 = P.t[2];
       const float fx = P.fx, fy = P.fy, cx = P.cx, cy = P.cy, Et = P.Et, Kb = P.Kb, cb = P.cb;
       const unsigned Wm2 = __float_as_uint(P.Wm2), Hm2 = __float_as_uint(P.Hm2);
+      constexpr int ILP = RPT < 2 ? RPT : 2;  // two samples in flight (four spill)
+      // the record of sample r of group g, as a multiple of blockDim past the thread's index
+      const auto at = [](int g, int r) { return HALVES == 2 ? g / 2 + 2 * r : g + r; };
       float acc[kAcc];
 #pragma unroll
       for (int k = 0; k < kAcc; ++k) acc[k] = 0.f;
-      constexpr int ILP = RPT < 2 ? RPT : 2;  // two samples in flight (four spill)
 #pragma unroll
       for (int g = 0; g < RPT; g += ILP) {
         float fu1[ILP], fv1[ILP], ca[ILP], cbf[ILP], xn[ILP], yn[ILP], iz[ILP], tb[ILP], dze[ILP];
         bool ok[ILP], fetch[ILP], amb[ILP];
 #pragma unroll
         for (int r = 0; r < ILP; ++r) {
-          const float4 X = s_X[threadIdx.x + (g + r) * blockDim.x];
+          const float4 X = s_X[threadIdx.x + at(g, r) * blockDim.x];
           // z, the largest component of X, enters last (rounded once), X0 and t first
           const float Y0 = fmaf(r2, X.z, fmaf(r1, X.y, fmaf(r0, X.x, t0)));
           const float Y1 = fmaf(r5, X.z, fmaf(r4, X.y, fmaf(r3, X.x, t1)));
@@ -767,7 +776,7 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
             base = __shfl_sync(0xffffffffu, base, leader);
             if (qa[r]) {
               const int pos = base + __popc(bal & lanemask_lt);
-              const int li = threadIdx.x + (g + r) * blockDim.x;
+              const int li = threadIdx.x + at(g, r) * blockDim.x;
               if (pos < kAmbCapPose) {
                 s_amb[pos] = AmbRef{td.begin + li, q, 0};
               } else {
@@ -809,10 +818,17 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
             }
           }
         }
+        // a7: warp reduce-scatter; lanes 0..7 store the warp's 8 sums (no block barrier)
+        if (HALVES == 2 || g + ILP >= RPT) {
+          const int row = warp + (HALVES == 2 ? g / 2 * nwarp : 0);
+          const float sred = warp_reduce_scatter8(acc, lane);
+          if (lane < 8) s_part[((size_t)row * a.max_pairs + (q - pb)) * kAcc + scatter_slot(lane)] = sred;
+          if (HALVES == 2) {
+#pragma unroll
+            for (int k = 0; k < kAcc; ++k) acc[k] = 0.f;
+          }
+        }
       }
-      // a7: warp reduce-scatter; lanes 0..7 store the warp's 8 sums (no block barrier)
-      const float sred = warp_reduce_scatter8(acc, lane);
-      if (lane < 8) s_part[((size_t)warp * a.max_pairs + (q - pb)) * kAcc + scatter_slot(lane)] = sred;
     }
     __syncthreads();  // every warp has stored its partial sums and appended its exact-path samples
     // the exact-path counts are read between the two barriers: every append of this tile is
@@ -826,7 +842,7 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
       const int2 pact = *reinterpret_cast<const int2*>(&a.pp[pb + qq].p);
       if (!pact.y) continue;
       float sum = 0.f;
-      for (int w = 0; w < nwarp; ++w) sum += s_part[((size_t)w * a.max_pairs + qq) * kAcc + slot];
+      for (int w = 0; w < HALVES * nwarp; ++w) sum += s_part[((size_t)w * a.max_pairs + qq) * kAcc + slot];
       if (sum != 0.f) atomicAdd(a.pair_acc + (size_t)kAcc * pact.x + slot, (double)sum);
     }
     if (threadIdx.x == 0) s_tile = s_next;
@@ -846,24 +862,24 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
   }
 }
 
-size_t edge_smem_bytes(int rpt, int block, int max_pairs, int refine) {
+size_t edge_smem_bytes(int rpt, int block, int max_pairs, int refine, int halves) {
   // dynamic part: lifted records, (refine scenes) their rays, per-warp per-pair partial sums
   return sizeof(float4) * (size_t)rpt * block +
          (refine ? sizeof(float2) * (size_t)rpt * block : 0) +
-         sizeof(float) * (refine ? edge_slots<1>() : edge_slots<0>()) * (size_t)max_pairs * (block / 32);
+         sizeof(float) * (refine ? edge_slots<1>() : edge_slots<0>()) * (size_t)max_pairs * halves * (block / 32);
 }
 
 // The kernel of a schedule: pose-only scenes run k_edge_pose, refine scenes k_edge.
-template <int MODE, int REC, int MAP, int GATHER, int R, int REF>
+template <int MODE, int REC, int MAP, int GATHER, int R, int REF, int HALVES = 1>
 static auto edge_kernel_of() {
   if constexpr (REF) return k_edge<MODE, REC, MAP, GATHER, R, 1>;
-  else return k_edge_pose<MODE, REC, MAP, GATHER, R>;
+  else return k_edge_pose<MODE, REC, MAP, GATHER, R, HALVES>;
 }
 
-template <int MODE, int REC, int MAP, int GATHER, int R, int REF>
+template <int MODE, int REC, int MAP, int GATHER, int R, int REF, int HALVES = 1>
 static cudaError_t launch_edge_one(const EdgeArgs& a, int block, int grid, cudaStream_t s) {
-  const size_t smem = edge_smem_bytes(R, block, a.max_pairs, REF);
-  const auto k = edge_kernel_of<MODE, REC, MAP, GATHER, R, REF>();
+  const size_t smem = edge_smem_bytes(R, block, a.max_pairs, REF, HALVES);
+  const auto k = edge_kernel_of<MODE, REC, MAP, GATHER, R, REF, HALVES>();
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -873,11 +889,16 @@ static cudaError_t launch_edge_one(const EdgeArgs& a, int block, int grid, cudaS
 
 // Refine scenes run two records per thread only (one set of instantiations).
 template <int MODE, int REC, int MAP, int GATHER, int REF>
-static cudaError_t launch_edge_rpt(const EdgeArgs& a, int rpt, int block, int grid, cudaStream_t s) {
+static cudaError_t launch_edge_rpt(const EdgeArgs& a, int rpt, int halves, int block, int grid, cudaStream_t s) {
   if constexpr (REF) {
-    if (rpt != 2) return cudaErrorInvalidValue;
+    if (rpt != 2 || halves != 1) return cudaErrorInvalidValue;
     return launch_edge_one<MODE, REC, MAP, GATHER, 2, 1>(a, block, grid, s);
   } else {
+    if (halves != 1) {
+      if constexpr (GATHER == GATHER_TEX)
+        if (halves == 2 && rpt == 4) return launch_edge_one<MODE, REC, MAP, GATHER, 4, 0, 2>(a, block, grid, s);
+      return cudaErrorInvalidValue;
+    }
     switch (rpt) {
       case 1: return launch_edge_one<MODE, REC, MAP, GATHER, 1, 0>(a, block, grid, s);
       case 2: return launch_edge_one<MODE, REC, MAP, GATHER, 2, 0>(a, block, grid, s);
@@ -889,48 +910,53 @@ static cudaError_t launch_edge_rpt(const EdgeArgs& a, int rpt, int block, int gr
 }
 
 template <int MODE, int REC, int MAP, int REF>
-static cudaError_t launch_edge_g(const EdgeArgs& a, int gather, int rpt, int block, int grid,
+static cudaError_t launch_edge_g(const EdgeArgs& a, int gather, int rpt, int halves, int block, int grid,
                                  cudaStream_t s) {
-  if (gather == GATHER_TEX) return launch_edge_rpt<MODE, REC, MAP, GATHER_TEX, REF>(a, rpt, block, grid, s);
+  if (gather == GATHER_TEX) return launch_edge_rpt<MODE, REC, MAP, GATHER_TEX, REF>(a, rpt, halves, block, grid, s);
   if constexpr (!REF) {
-    if (gather == GATHER_MIX) return launch_edge_rpt<MODE, REC, MAP, GATHER_MIX, REF>(a, rpt, block, grid, s);
+    if (gather == GATHER_MIX) return launch_edge_rpt<MODE, REC, MAP, GATHER_MIX, REF>(a, rpt, halves, block, grid, s);
   }
   if (gather != GATHER_LDG) return cudaErrorInvalidValue;
-  return launch_edge_rpt<MODE, REC, MAP, GATHER_LDG, REF>(a, rpt, block, grid, s);
+  return launch_edge_rpt<MODE, REC, MAP, GATHER_LDG, REF>(a, rpt, halves, block, grid, s);
 }
 
 template <int MODE, int REF>
-static cudaError_t launch_edge_m(const EdgeArgs& a, int rec, int map, int gather, int rpt, int block,
+static cudaError_t launch_edge_m(const EdgeArgs& a, int rec, int map, int gather, int rpt, int halves, int block,
                                  int grid, cudaStream_t s) {
-  if (rec == 0 && map == 0) return launch_edge_g<MODE, 0, 0, REF>(a, gather, rpt, block, grid, s);
-  if (rec == 0 && map == 1) return launch_edge_g<MODE, 0, 1, REF>(a, gather, rpt, block, grid, s);
-  if (rec == 1 && map == 0) return launch_edge_g<MODE, 1, 0, REF>(a, gather, rpt, block, grid, s);
-  return launch_edge_g<MODE, 1, 1, REF>(a, gather, rpt, block, grid, s);
+  if (rec == 0 && map == 0) return launch_edge_g<MODE, 0, 0, REF>(a, gather, rpt, halves, block, grid, s);
+  if (rec == 0 && map == 1) return launch_edge_g<MODE, 0, 1, REF>(a, gather, rpt, halves, block, grid, s);
+  if (rec == 1 && map == 0) return launch_edge_g<MODE, 1, 0, REF>(a, gather, rpt, halves, block, grid, s);
+  return launch_edge_g<MODE, 1, 1, REF>(a, gather, rpt, halves, block, grid, s);
 }
 
 template <int MODE>
-static cudaError_t launch_edge_r(const EdgeArgs& a, int refine, int rec, int map, int gather, int rpt, int block,
-                                 int grid, cudaStream_t s) {
-  if (refine) return launch_edge_m<MODE, 1>(a, rec, map, gather, rpt, block, grid, s);
-  return launch_edge_m<MODE, 0>(a, rec, map, gather, rpt, block, grid, s);
+static cudaError_t launch_edge_r(const EdgeArgs& a, int refine, int rec, int map, int gather, int rpt, int halves,
+                                 int block, int grid, cudaStream_t s) {
+  if (refine) return launch_edge_m<MODE, 1>(a, rec, map, gather, rpt, halves, block, grid, s);
+  return launch_edge_m<MODE, 0>(a, rec, map, gather, rpt, halves, block, grid, s);
 }
 
 // rec_dtype: 0 = f32 records, 1 = f16-depth records; map_dtype: 0 = f32, 1 = bf16.
 cudaError_t launch_edge(const EdgeArgs& a, int mode, int refine, int rec_dtype, int map_dtype, int gather,
-                        int rpt, int block, int grid, cudaStream_t s) {
+                        int rpt, int halves, int block, int grid, cudaStream_t s) {
   if (a.n_tiles == 0) return cudaSuccess;
   switch (mode) {
-    case MODE_FWD: return launch_edge_r<MODE_FWD>(a, refine, rec_dtype, map_dtype, gather, rpt, block, grid, s);
-    case MODE_BWD: return launch_edge_r<MODE_BWD>(a, refine, rec_dtype, map_dtype, gather, rpt, block, grid, s);
-    default: return launch_edge_r<MODE_FUSED>(a, refine, rec_dtype, map_dtype, gather, rpt, block, grid, s);
+    case MODE_FWD: return launch_edge_r<MODE_FWD>(a, refine, rec_dtype, map_dtype, gather, rpt, halves, block, grid, s);
+    case MODE_BWD: return launch_edge_r<MODE_BWD>(a, refine, rec_dtype, map_dtype, gather, rpt, halves, block, grid, s);
+    default: return launch_edge_r<MODE_FUSED>(a, refine, rec_dtype, map_dtype, gather, rpt, halves, block, grid, s);
   }
 }
 
 template <int MODE, int REC, int MAP, int GATHER, int REF>
-static const void* edge_ptr_rpt(int rpt) {
+static const void* edge_ptr_rpt(int rpt, int halves) {
   if constexpr (REF) {
-    return rpt == 2 ? (const void*)k_edge<MODE, REC, MAP, GATHER, 2, 1> : nullptr;
+    return rpt == 2 && halves == 1 ? (const void*)k_edge<MODE, REC, MAP, GATHER, 2, 1> : nullptr;
   } else {
+    if (halves != 1) {
+      if constexpr (GATHER == GATHER_TEX)
+        if (halves == 2 && rpt == 4) return (const void*)edge_kernel_of<MODE, REC, MAP, GATHER, 4, 0, 2>();
+      return nullptr;
+    }
     switch (rpt) {
       case 1: return (const void*)edge_kernel_of<MODE, REC, MAP, GATHER, 1, 0>();
       case 2: return (const void*)edge_kernel_of<MODE, REC, MAP, GATHER, 2, 0>();
@@ -942,40 +968,40 @@ static const void* edge_ptr_rpt(int rpt) {
 }
 
 template <int MODE, int REF>
-static const void* edge_ptr_m(int rec, int map, int gather, int rpt) {
+static const void* edge_ptr_m(int rec, int map, int gather, int rpt, int halves) {
   if constexpr (!REF) {
     if (gather == GATHER_MIX) {
-      if (rec == 0 && map == 0) return edge_ptr_rpt<MODE, 0, 0, GATHER_MIX, REF>(rpt);
-      if (rec == 0 && map == 1) return edge_ptr_rpt<MODE, 0, 1, GATHER_MIX, REF>(rpt);
-      if (rec == 1 && map == 0) return edge_ptr_rpt<MODE, 1, 0, GATHER_MIX, REF>(rpt);
-      return edge_ptr_rpt<MODE, 1, 1, GATHER_MIX, REF>(rpt);
+      if (rec == 0 && map == 0) return edge_ptr_rpt<MODE, 0, 0, GATHER_MIX, REF>(rpt, halves);
+      if (rec == 0 && map == 1) return edge_ptr_rpt<MODE, 0, 1, GATHER_MIX, REF>(rpt, halves);
+      if (rec == 1 && map == 0) return edge_ptr_rpt<MODE, 1, 0, GATHER_MIX, REF>(rpt, halves);
+      return edge_ptr_rpt<MODE, 1, 1, GATHER_MIX, REF>(rpt, halves);
     }
   }
   if (gather == GATHER_MIX) return nullptr;
   if (gather == GATHER_TEX) {
-    if (rec == 0 && map == 0) return edge_ptr_rpt<MODE, 0, 0, GATHER_TEX, REF>(rpt);
-    if (rec == 0 && map == 1) return edge_ptr_rpt<MODE, 0, 1, GATHER_TEX, REF>(rpt);
-    if (rec == 1 && map == 0) return edge_ptr_rpt<MODE, 1, 0, GATHER_TEX, REF>(rpt);
-    return edge_ptr_rpt<MODE, 1, 1, GATHER_TEX, REF>(rpt);
+    if (rec == 0 && map == 0) return edge_ptr_rpt<MODE, 0, 0, GATHER_TEX, REF>(rpt, halves);
+    if (rec == 0 && map == 1) return edge_ptr_rpt<MODE, 0, 1, GATHER_TEX, REF>(rpt, halves);
+    if (rec == 1 && map == 0) return edge_ptr_rpt<MODE, 1, 0, GATHER_TEX, REF>(rpt, halves);
+    return edge_ptr_rpt<MODE, 1, 1, GATHER_TEX, REF>(rpt, halves);
   }
-  if (rec == 0 && map == 0) return edge_ptr_rpt<MODE, 0, 0, GATHER_LDG, REF>(rpt);
-  if (rec == 0 && map == 1) return edge_ptr_rpt<MODE, 0, 1, GATHER_LDG, REF>(rpt);
-  if (rec == 1 && map == 0) return edge_ptr_rpt<MODE, 1, 0, GATHER_LDG, REF>(rpt);
-  return edge_ptr_rpt<MODE, 1, 1, GATHER_LDG, REF>(rpt);
+  if (rec == 0 && map == 0) return edge_ptr_rpt<MODE, 0, 0, GATHER_LDG, REF>(rpt, halves);
+  if (rec == 0 && map == 1) return edge_ptr_rpt<MODE, 0, 1, GATHER_LDG, REF>(rpt, halves);
+  if (rec == 1 && map == 0) return edge_ptr_rpt<MODE, 1, 0, GATHER_LDG, REF>(rpt, halves);
+  return edge_ptr_rpt<MODE, 1, 1, GATHER_LDG, REF>(rpt, halves);
 }
 
-const void* edge_kernel_ptr(int mode, int refine, int rec_dtype, int map_dtype, int gather, int rpt) {
+const void* edge_kernel_ptr(int mode, int refine, int rec_dtype, int map_dtype, int gather, int rpt, int halves) {
   if (refine) {
     switch (mode) {
-      case MODE_FWD: return edge_ptr_m<MODE_FWD, 1>(rec_dtype, map_dtype, gather, rpt);
-      case MODE_BWD: return edge_ptr_m<MODE_BWD, 1>(rec_dtype, map_dtype, gather, rpt);
-      default: return edge_ptr_m<MODE_FUSED, 1>(rec_dtype, map_dtype, gather, rpt);
+      case MODE_FWD: return edge_ptr_m<MODE_FWD, 1>(rec_dtype, map_dtype, gather, rpt, halves);
+      case MODE_BWD: return edge_ptr_m<MODE_BWD, 1>(rec_dtype, map_dtype, gather, rpt, halves);
+      default: return edge_ptr_m<MODE_FUSED, 1>(rec_dtype, map_dtype, gather, rpt, halves);
     }
   }
   switch (mode) {
-    case MODE_FWD: return edge_ptr_m<MODE_FWD, 0>(rec_dtype, map_dtype, gather, rpt);
-    case MODE_BWD: return edge_ptr_m<MODE_BWD, 0>(rec_dtype, map_dtype, gather, rpt);
-    default: return edge_ptr_m<MODE_FUSED, 0>(rec_dtype, map_dtype, gather, rpt);
+    case MODE_FWD: return edge_ptr_m<MODE_FWD, 0>(rec_dtype, map_dtype, gather, rpt, halves);
+    case MODE_BWD: return edge_ptr_m<MODE_BWD, 0>(rec_dtype, map_dtype, gather, rpt, halves);
+    default: return edge_ptr_m<MODE_FUSED, 0>(rec_dtype, map_dtype, gather, rpt, halves);
   }
 }
 

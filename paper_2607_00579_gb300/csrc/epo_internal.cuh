@@ -342,7 +342,7 @@ cudaError_t launch_mlp_update(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_depth(const StepArgs& a, int update, cudaStream_t s);
 cudaError_t launch_l2_read(const void* p, int64_t bytes, unsigned* sink, int sms, cudaStream_t s);
 cudaError_t launch_edge(const EdgeArgs& a, int mode, int refine, int rec_dtype, int map_dtype, int gather,
-                        int rpt, int block, int grid, cudaStream_t s);
+                        int rpt, int halves, int block, int grid, cudaStream_t s);
 // pose kernel: with_grad 0 = loss only, 1 = loss + gradient, 2 = + Adam/Exp update
 cudaError_t launch_poses(const StepArgs& a, int with_grad, cudaStream_t s);
 // A launch that allows programmatic dependent launch on stream s (see griddep_wait).
@@ -375,7 +375,7 @@ cudaError_t launch_round_bf16(const float* src, uint16_t* dst, int64_t n, cudaSt
 cudaError_t launch_lift_records(const void* rec, int rec_dtype, const ViewDev* views, const double* K64,
                                 int n_views, float eps_z, float4* out, cudaStream_t s);
 int edt_max_height();
-const void* edge_kernel_ptr(int mode, int refine, int rec_dtype, int map_dtype, int gather, int rpt);
-size_t edge_smem_bytes(int rpt, int block, int max_pairs, int refine);
+const void* edge_kernel_ptr(int mode, int refine, int rec_dtype, int map_dtype, int gather, int rpt, int halves);
+size_t edge_smem_bytes(int rpt, int block, int max_pairs, int refine, int halves);
 
 }  // namespace epo

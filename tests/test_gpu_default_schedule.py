@@ -1,4 +1,4 @@
-"""The default schedule against explicit ones on the same scene.  The sums of a work item are formed
+"""The default schedule against plain loads in the 256-thread form, unsplit, on the same scene.  The sums of a work item are formed
 in one order whatever the gather path and the split of its pairs, so the results agree to the order
 of FP64 atomics (1e-12 leaves four digits for cancellation in the gradient)."""
 import numpy as np
@@ -41,15 +41,22 @@ def evaluate(s, refine):
     if refine:
         i = s.info()
         return B.epo_refine_loss_and_grad(s.handle, i.n_scenes, i.n_views, i.n_records)
-    return (*s.loss_and_grad(), s.pair_stats())
+    out = (*s.loss_and_grad(), s.pair_stats())
+    xi = torch.full((s.n_views, 6), 1e-3, dtype=torch.float64, device="cuda", requires_grad=True)
+    loss = epo.EdgeLoss.apply(xi, s)  # the forward-only and adjoint-only kernels
+    (grad,) = torch.autograd.grad(loss.sum(), xi)
+    return (*out, loss.detach().cpu().numpy(), grad.cpu().numpy())
 
 
 @pytest.mark.parametrize("W,H,n_views,n_rec,k", [(2, 2, 2, 9, 1), (3, 65, 3, 700, 2), (64, 48, 5, 513, 4),
-                                                 (161, 123, 12, 1500, 11), (97, 80, 40, 5000, 8)])
+                                                 (161, 123, 12, 1500, 11), (97, 80, 40, 5000, 8),
+                                                 (80, 60, 130, 2600, 9)])
 @pytest.mark.parametrize("mixed", [False, True])
 @pytest.mark.parametrize("refine", [0, 1])
 def test_default_equals_plain_loads(W, H, n_views, n_rec, k, mixed, refine):
     a = scene(W, H, n_views, n_rec, k, mixed, refine=refine)
+    if n_views == 130 and not refine:  # enough work for the 128-thread form of the default item
+        assert (a.info().block_threads, a.info().records_per_thread) == (128, 4)
     b = scene(W, H, n_views, n_rec, k, mixed, refine=refine, gather=epo.EPO_GATHER_LDG, tail_pairs=0)
     assert (a.info().gather, b.info().gather) == (epo.EPO_GATHER_TEX, epo.EPO_GATHER_LDG)
     for x, y in zip(evaluate(a, refine), evaluate(b, refine)):
