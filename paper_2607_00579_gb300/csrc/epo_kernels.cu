@@ -188,6 +188,7 @@ __device__ __forceinline__ double cross_entry(int r, int c, double w0, double w1
 
 __global__ void __launch_bounds__(kPoseThreads) k_poses(StepArgs a, int with_grad, int n_pose_blocks) {
   static_assert(kPoseThreads == 32 && kLossChunk == 32, "one warp per block, one pair per lane");
+  griddep_launch_dependents();  // the pose MLP's backward kernel starts on its weights
   const int64_t step = *a.step;
   int flag0 = *a.flag;
   bool bad_here = false;  // this thread set the non-finite flag in this step
