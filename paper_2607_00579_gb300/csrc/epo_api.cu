@@ -575,28 +575,35 @@ bool schedule_fits(epo_scene* S, const Sched& sc) {
   return (!S->refine || sc.rpt == 2) && edge_smem_bytes(sc.rpt, sc.block, item_pairs(S, sc), S->refine, sc.halves) <= kMaxSmem;
 }
 
-// The schedule of a pose-only scene whose options leave it to the library.  All of these give the
-// same bits: a work item is 512 records, either two per thread of 256 threads or four per thread of
-// 128 (two halves, k_edge_pose), and a split by pairs moves whole sums to other blocks.
+// What the options leave to the library of a scene's schedule (texture gather, the library's grid).  A
+// split by pairs moves whole sums to other blocks, and the two forms of the default item (512 records,
+// two per thread of 256 threads or four per thread of 128 in two halves, k_edge_pose) form the same
+// sums, so all of these give the same bits as the unsplit 256-thread form.
 //
-// With U = work items x pairs (those a step evaluates) and G = 1368 resident 128-thread blocks:
-//  - U >= 4 G: 128 threads, items of about sqrt(U / 2G) pairs.  On a full SM a pair of one item
-//    takes ~3.6 us, so a block that claims a whole item last keeps the others waiting; each item
-//    costs about a quarter of a pair more.  U / G + U / (4 G n) + n / 2 is least there.  Once that
-//    nears the whole item nothing is split.
-//  - below, 256 threads: one wave of items if at most 4 pairs each make one (a block that runs alone
-//    is bound by the latency of its pairs, one after the other); else items of 4 where the whole ones
-//    fill the SMs or are longer than 8.
+// With U = work items x pairs (those a step evaluates) and G = the resident 128-thread blocks:
+//  - no block size given and U < 4 G: 256 threads; one wave of items if at most 4 pairs each make one
+//    (a block that runs alone is bound by the latency of its pairs, one after the other), else items
+//    of 4 where the whole ones fill the SMs or are longer than 8.
+//  - otherwise, and for 128 threads with four records given: items of about sqrt(U / 2G) pairs.  On a
+//    full SM a pair of one item takes ~3.6 us, so a block that claims a whole item last keeps the
+//    others waiting; each item costs about a quarter of a pair more.  U / G + U / (4 G n) + n / 2 is
+//    least there.  From U = 36 G on whole items, the last wave's in twos.
+//  - with refinement (256 threads): one wave of items as above; between one and two waves, the last
+//    one's in halves.
 // Step, microseconds, 256 threads unsplit -> this rule: 8 views of 128x96 all pairs 24.8 -> 18.6;
-// 14 of 319x241 35.3 -> 24.8; 32 of 256x192 29.6 -> 22.6; 30 of 518x392 with 12
-// pairs a view 39.1 -> 33.0; 16 of 518x392 30.5, not split (31.0 in fours); 120 of 256x192 46.7 ->
-// 37.3; 32 of 518x392 51.1 -> 49.2; 48 of 518x392 67.4 -> 65.6; 20 of 518x518 all pairs, BF16
-// 88.6 -> 75.0; 96 of 518x392 92.8 -> 82.7; 120 of 518x392 157 -> 147; 200 of 518x392 333 -> 311; 300 of
-// 518x518, BF16 652 -> 594; 24 uneven scenes 689 -> 625.
+// 14 of 319x241 35.3 -> 24.8; 32 of 256x192 29.6 -> 22.6; 30 of 518x392 with 12 pairs a view 39.1 ->
+// 33.0; 16 of 518x392 30.5, not split (31.0 in fours); 120 of 256x192 46.7 -> 37.3; 32 of 518x392 51.1
+// -> 49.2; 48 of 518x392 67.4 -> 65.6; 20 of 518x518 all pairs, BF16 88.6 -> 75.0; 96 of 518x392 92.8 ->
+// 82.7; 120 of 518x392 157 -> 147; 200 of 518x392 333 -> 311; 300 of 518x518, BF16 652 -> 587; 24 uneven
+// scenes 689 -> 620.  128 threads and four records given, unsplit -> this rule: 48 of 518x392 76.0 ->
+// 62.0; 64 of 518x518, BF16 118 -> 111; 96 of 518x518, BF16 165 -> 152; 200 of 518x392 283 -> 277.  With
+// refinement: 24 of 256x192 45.7 -> 37.1; 32 of 518x392 77.0 -> 71.9; 64 of 518x392 148, not split.
 void default_schedule(epo_scene* S) {
-  const Sched wide = S->sch;  // 256 threads, two records per thread
-  if (wide.block != 256 || wide.rpt != 2) return;
-  const double G = 1368.0;
+  const epo_options& o = S->opt;
+  const bool open = o.block_threads == 0 && o.records_per_thread == 0;
+  if (S->sch.gather != GATHER_TEX || o.grid_blocks != 0 || o.tail_pairs != -1) return;
+  if (!(open && S->sch.block == 256 && S->sch.rpt == 2) && !(!S->refine && S->sch.block == 128 && S->sch.rpt == 4)) return;
+  const double G = 9.0 * S->sm_count, wide_slots = 4.0 * S->sm_count;
   double tiles = 0.0, U = 0.0;
   for (int v = 0; v < S->n_views; ++v) {
     const int k = S->src_pair_off[v + 1] - S->src_pair_off[v];
@@ -606,35 +613,41 @@ void default_schedule(epo_scene* S) {
   }
   if (!(U > 0.0)) return;
   double share = 1.0;  // of the pairs a step evaluates (Algorithm 3's budget)
-  if (S->opt.pair_budget > 0) {
+  if (o.pair_budget > 0) {
     double act = 0.0;
     for (int sc = 0; sc < S->n_scenes; ++sc)
-      act += std::min(S->opt.pair_budget, S->scene_pair_off[sc + 1] - S->scene_pair_off[sc]);
+      act += std::min(o.pair_budget, S->scene_pair_off[sc + 1] - S->scene_pair_off[sc]);
     share = act / S->n_pairs;
   }
-  const double k = U / tiles;  // pairs per view
-  if (U * share >= 4.0 * G) {
-    S->sch.block = 128;
-    S->sch.rpt = 4;
-    S->sch.halves = 2;
-    const double n = std::max(1.0, floor(sqrt(U * share / (2.0 * G)) / share + 0.5));
-    const double even = ceil(k / ceil(k / n));  // pieces of equal size
-    if (n < 0.75 * k) S->sch.tail = -(int)even;
-    if (!schedule_fits(S, S->sch)) S->sch = wide;
+  const double k = U / tiles, u = U * share / G;
+  if (!S->refine && (!open || u >= 4.0)) {
+    Sched sc = S->sch;
+    if (open) {
+      sc.block = 128;
+      sc.rpt = 4;
+      sc.halves = 2;
+    }
+    if (u >= 36.0) {
+      sc.tail = (int)ceil(2.0 / share);
+    } else {
+      const double n = std::max(1.0, floor(sqrt(u / 2.0) / share + 0.5));
+      if (n < k) sc.tail = -(int)ceil(k / ceil(k / n));  // pieces of equal size
+    }
+    if (schedule_fits(S, sc)) S->sch = sc;
     return;
   }
-  const double slots = S->sm_count * 4.0;
   for (int n = 1; n <= 4 && n < S->max_pairs; ++n) {
     double items = 0.0;
     for (int v = 0; v < S->n_views; ++v) {
       const int kv = S->src_pair_off[v + 1] - S->src_pair_off[v];
       items += (double)((S->views[v].n_rec + 511) / 512) * ((kv + n - 1) / n);
     }
-    if (items <= slots || (n == 4 && (k > 8.0 || tiles > 0.9 * slots))) {
+    if (items <= wide_slots || (!S->refine && n == 4 && (k > 8.0 || tiles > 0.9 * wide_slots))) {
       S->sch.tail = -n;
       return;
     }
   }
+  if (S->refine && tiles > wide_slots && tiles < 2.0 * wide_slots) S->sch.tail = (int)ceil(k / 2.0);
 }
 
 // Record stage event k on stream s (inside a capture it becomes an event-record node).
@@ -1288,9 +1301,7 @@ epo_status create_impl(int32_t n_scenes, const epo_scene_desc* descs, const epo_
     S->sch.gather = o.gather == EPO_GATHER_LDG ? GATHER_LDG : (o.gather == EPO_GATHER_MIX ? GATHER_MIX : GATHER_TEX);
     if (!schedule_fits(S, S->sch)) S->sch.block = 128;
     S->sch.tail = o.tail_pairs == -1 ? 0 : o.tail_pairs;
-    if (!S->refine && S->sch.gather == GATHER_TEX && o.block_threads == 0 && o.records_per_thread == 0 &&
-        o.grid_blocks == 0 && o.tail_pairs == -1)
-      default_schedule(S);
+    default_schedule(S);
     epo_status bs = build_tiles(S);
     if (bs != EPO_OK) return bs;
     CK(cudaStreamSynchronize(st));

@@ -61,3 +61,21 @@ def test_default_equals_plain_loads(W, H, n_views, n_rec, k, mixed, refine):
     assert (a.info().gather, b.info().gather) == (epo.EPO_GATHER_TEX, epo.EPO_GATHER_LDG)
     for x, y in zip(evaluate(a, refine), evaluate(b, refine)):
         assert np.abs(x - y).max() <= 1e-12 * max(np.abs(y).max(), 1e-300)
+
+
+@pytest.mark.parametrize("W,H,n_views,n_rec,k", [(64, 48, 5, 513, 4), (97, 80, 40, 5000, 8), (80, 60, 130, 2600, 9),
+                                                 (32, 24, 330, 4100, 18)])
+@pytest.mark.parametrize("opt", [dict(), dict(pair_budget=37, subsample_seed=3), dict(refine=1)])
+def test_split_items_equal_whole_ones(W, H, n_views, n_rec, k, opt):
+    """The library's split of the items (also the last wave's alone, the largest scene here) against
+    whole items, for the default schedule and for 128 threads with four records each."""
+    for sched in (dict(), dict(gather=epo.EPO_GATHER_TEX, block_threads=128, records_per_thread=4)):
+        if sched and "refine" in opt:
+            continue
+        a = scene(W, H, n_views, n_rec, k, False, **opt, **sched)
+        whole = sched or dict(gather=epo.EPO_GATHER_TEX, block_threads=256, records_per_thread=2)
+        if "refine" in opt:
+            whole = dict(gather=epo.EPO_GATHER_TEX)
+        b = scene(W, H, n_views, n_rec, k, False, tail_pairs=0, **opt, **whole)
+        for x, y in zip(evaluate(a, "refine" in opt), evaluate(b, "refine" in opt)):
+            assert np.abs(x - y).max() <= 1e-12 * max(np.abs(y).max(), 1e-300)
