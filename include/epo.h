@@ -251,6 +251,14 @@ epo_status epo_forward_dev(epo_scene_t scene, const double* xi_dev, double* loss
 epo_status epo_backward_dev(epo_scene_t scene, const double* xi_dev, const double* dloss_dev,
                             double* grad_xi_dev);
 
+/* The same function with one pass over the samples: forward_grad also forms g, the left-perturbation
+ * gradient at T(xi) of every view's scene loss (n_views x 6, device, the caller's), and
+ * backward_from turns it into d(out)/d(xi) = J_l(xi)^T (dloss g).  g holds all that the backward
+ * needs, so other evaluations may come between the two. */
+epo_status epo_forward_grad_dev(epo_scene_t scene, const double* xi_dev, double* loss_dev, double* grad_dev);
+epo_status epo_backward_from_dev(epo_scene_t scene, const double* xi_dev, const double* grad_dev,
+                                 const double* dloss_dev, double* grad_xi_dev);
+
 /* n_steps optimisation steps (Algorithm 2, pose-only reading): clamp anneal,
  * loss + gradient, tangent-space Adam, T_i <- Exp(-Delta_i) T_i for every
  * view not fixed.  Each step is one replay of a CUDA graph; lambda, the step

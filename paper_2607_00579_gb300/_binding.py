@@ -41,7 +41,7 @@ EXPORTED = [
     "epo_loss_and_grad_noalloc", "epo_gather_probe", "epo_set_refinement", "epo_refine_loss_and_grad",
     "epo_get_pair_active", "epo_get_schedule", "epo_build_viewgraph", "epo_get_refinement",
     "epo_set_pose_mlp", "epo_get_pose_mlp", "epo_get_pose_mlp_moments", "epo_step_host",
-    "epo_set_wait_limit",
+    "epo_set_wait_limit", "epo_forward_grad_dev", "epo_backward_from_dev",
 ]
 
 
@@ -141,6 +141,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
         "epo_pair_stats": (I32, [S, P]),
         "epo_forward_dev": (I32, [S, P, P]),
         "epo_backward_dev": (I32, [S, P, P, P]),
+        "epo_forward_grad_dev": (I32, [S, P, P, P]),
+        "epo_backward_from_dev": (I32, [S, P, P, P, P]),
         "epo_step": (I32, [S, I32]),
         "epo_step_async": (I32, [S, I32]),
         "epo_step_plain": (I32, [S, I32]),
@@ -240,6 +242,8 @@ def epo_loss_and_grad_dev(scene, loss, grad): _call("epo_loss_and_grad_dev", sce
 def epo_pair_stats(scene, stats): _call("epo_pair_stats", scene, _ptr(stats))
 def epo_forward_dev(scene, xi, loss): _call("epo_forward_dev", scene, _ptr(xi), _ptr(loss))
 def epo_backward_dev(scene, xi, dloss, grad): _call("epo_backward_dev", scene, _ptr(xi), _ptr(dloss), _ptr(grad))
+def epo_forward_grad_dev(scene, xi, loss, grad): _call("epo_forward_grad_dev", scene, _ptr(xi), _ptr(loss), _ptr(grad))
+def epo_backward_from_dev(scene, xi, grad, dloss, gxi): _call("epo_backward_from_dev", scene, _ptr(xi), _ptr(grad), _ptr(dloss), _ptr(gxi))
 def epo_step(scene, n): _call("epo_step", scene, ctypes.c_int32(n))
 def epo_step_async(scene, n): _call("epo_step_async", scene, ctypes.c_int32(n))
 def epo_step_plain(scene, n): _call("epo_step_plain", scene, ctypes.c_int32(n))

@@ -1620,22 +1620,28 @@ epo_status epo_pair_stats(epo_scene_t S, double* stats) {
   return EPO_OK;
 }
 
+// One evaluation at Exp(xi) T on the scene's stream: pair setup, edge kernel, pose kernel.
+static epo_status enqueue_at_twists(epo_scene* S, const double* xi_dev, StepArgs a, int mode, int with_grad) {
+  CK(launch_twist_poses(S->d_T, xi_dev, S->d_T_eval, S->n_views, S->stream));
+  MARK(0, S->stream);
+  if (S->subsample) CK(launch_subsample(a, S->stream));
+  if (S->refine) CK(launch_refine_intrinsics(a, S->stream));
+  CK(launch_pair_setup(a, mode, S->stream));
+  MARK(1, S->stream);
+  epo_status st = run_edge(S, mode, S->sch, S->stream);
+  if (st != EPO_OK) return st;
+  CK(launch_poses(a, with_grad, S->stream));
+  MARK(3, S->stream);
+  return EPO_OK;
+}
+
 epo_status epo_forward_dev(epo_scene_t S, const double* xi_dev, double* loss_dev) {
   EPO_RANGE("epo_forward_dev");
   if (!S || !loss_dev) return fail(S, EPO_ERR_INVALID_ARG, "null argument");
   epo_status st = maybe_autotune(S);
   if (st != EPO_OK) return st;
-  CK(launch_twist_poses(S->d_T, xi_dev, S->d_T_eval, S->n_views, S->stream));
-  StepArgs a = step_args(S, S->d_T_eval, nullptr);
-  MARK(0, S->stream);
-  if (S->subsample) CK(launch_subsample(a, S->stream));
-  if (S->refine) CK(launch_refine_intrinsics(a, S->stream));
-  CK(launch_pair_setup(a, MODE_FWD, S->stream));
-  MARK(1, S->stream);
-  st = run_edge(S, MODE_FWD, S->sch, S->stream);
+  st = enqueue_at_twists(S, xi_dev, step_args(S, S->d_T_eval, nullptr), MODE_FWD, 0);
   if (st != EPO_OK) return st;
-  CK(launch_poses(a, 0, S->stream));
-  MARK(3, S->stream);
   CK(cudaMemcpyAsync(loss_dev, S->d_loss, (size_t)S->n_scenes * 8, cudaMemcpyDeviceToDevice, S->stream));
   return EPO_OK;
 }
@@ -1644,18 +1650,28 @@ epo_status epo_backward_dev(epo_scene_t S, const double* xi_dev, const double* d
                             double* grad_xi_dev) {
   EPO_RANGE("epo_backward_dev");
   if (!S || !dloss_dev || !grad_xi_dev) return fail(S, EPO_ERR_INVALID_ARG, "null argument");
-  CK(launch_twist_poses(S->d_T, xi_dev, S->d_T_eval, S->n_views, S->stream));
-  StepArgs a = step_args(S, S->d_T_eval, dloss_dev);
-  MARK(0, S->stream);
-  if (S->subsample) CK(launch_subsample(a, S->stream));
-  if (S->refine) CK(launch_refine_intrinsics(a, S->stream));
-  CK(launch_pair_setup(a, MODE_BWD, S->stream));
-  MARK(1, S->stream);
-  epo_status st = run_edge(S, MODE_BWD, S->sch, S->stream);
+  epo_status st = enqueue_at_twists(S, xi_dev, step_args(S, S->d_T_eval, dloss_dev), MODE_BWD, 1);
   if (st != EPO_OK) return st;
-  CK(launch_poses(a, 1, S->stream));
-  MARK(3, S->stream);
-  CK(launch_apply_left_jacobian(xi_dev, S->d_grad, grad_xi_dev, S->n_views, S->stream));
+  CK(launch_apply_left_jacobian(xi_dev, S->d_grad, grad_xi_dev, S->n_views, nullptr, S->d_views, S->d_flag, S->stream));
+  return EPO_OK;
+}
+
+epo_status epo_forward_grad_dev(epo_scene_t S, const double* xi_dev, double* loss_dev, double* grad_dev) {
+  EPO_RANGE("epo_forward_grad_dev");
+  if (!S || !loss_dev || !grad_dev) return fail(S, EPO_ERR_INVALID_ARG, "null argument");
+  epo_status st = maybe_autotune(S);
+  if (st != EPO_OK) return st;
+  StepArgs a = step_args(S, S->d_T_eval, nullptr);
+  a.loss_out = loss_dev;
+  a.grad = grad_dev;
+  return enqueue_at_twists(S, xi_dev, a, MODE_FUSED, 1);
+}
+
+epo_status epo_backward_from_dev(epo_scene_t S, const double* xi_dev, const double* grad_dev, const double* dloss_dev,
+                                 double* grad_xi_dev) {
+  EPO_RANGE("epo_backward_from_dev");
+  if (!S || !grad_dev || !dloss_dev || !grad_xi_dev) return fail(S, EPO_ERR_INVALID_ARG, "null argument");
+  CK(launch_apply_left_jacobian(xi_dev, grad_dev, grad_xi_dev, S->n_views, dloss_dev, S->d_views, S->d_flag, S->stream));
   return EPO_OK;
 }
 

@@ -240,6 +240,7 @@ struct StepArgs {
   double* pair_acc;
   double* grad;                      // n_views x 6
   double* loss;                      // n_scenes
+  double* loss_out;                  // a caller's copy of it (NULL if unused)
   double* m;                         // Adam moments
   double* v;
   double* bpow;                      // beta1^(s+1), beta2^(s+1) for the next step s
@@ -365,8 +366,10 @@ inline cudaError_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, si
 cudaError_t launch_io_copy(const double* src, double* dst, int64_t n, cudaStream_t s);
 cudaError_t launch_twist_poses(const double* T, const double* xi, double* T_out, int n,
                                cudaStream_t s);
-cudaError_t launch_apply_left_jacobian(const double* xi, const double* g, double* out, int n,
-                                       cudaStream_t s);
+// out = J_l(xi)^T (scale g); scale: dloss of the view's scene (NULL = 1).  A non-finite scaled gradient
+// sets the status word, as it does in the pose kernel.
+cudaError_t launch_apply_left_jacobian(const double* xi, const double* g, double* out, int n, const double* dloss,
+                                       const ViewDev* views, int32_t* flag, cudaStream_t s);
 cudaError_t launch_map_check(const void* map, int dtype, int64_t n, int32_t* bad, cudaStream_t s);
 cudaError_t launch_edt(const uint8_t* edges, int W, int H, float* map, cudaStream_t s);
 cudaError_t launch_round_bf16(const float* src, uint16_t* dst, int64_t n, cudaStream_t s);

@@ -42,10 +42,11 @@ def evaluate(s, refine):
         i = s.info()
         return B.epo_refine_loss_and_grad(s.handle, i.n_scenes, i.n_views, i.n_records)
     out = (*s.loss_and_grad(), s.pair_stats())
-    xi = torch.full((s.n_views, 6), 1e-3, dtype=torch.float64, device="cuda", requires_grad=True)
-    loss = epo.EdgeLoss.apply(xi, s)  # the forward-only and adjoint-only kernels
-    (grad,) = torch.autograd.grad(loss.sum(), xi)
-    return (*out, loss.detach().cpu().numpy(), grad.cpu().numpy())
+    xi = torch.full((s.n_views, 6), 1e-3, dtype=torch.float64, device="cuda")  # forward-only and adjoint-only
+    loss, grad = torch.empty(1, dtype=torch.float64, device="cuda"), torch.empty_like(xi)
+    B.epo_forward_dev(s.handle, xi, loss)
+    B.epo_backward_dev(s.handle, xi, torch.ones_like(loss), grad)
+    return (*out, loss.cpu().numpy(), grad.cpu().numpy())
 
 
 @pytest.mark.parametrize("W,H,n_views,n_rec,k", [(2, 2, 2, 9, 1), (3, 65, 3, 700, 2), (64, 48, 5, 513, 4),
