@@ -29,8 +29,13 @@ def library_path() -> str:
 
 
 def _current_stream() -> int:
+    """The raw handle of torch's current stream (without a Stream object around it where torch has
+    that: 0.4 us instead of 3, a fifth of the host's share of a small call)."""
     import torch
-    return torch.cuda.current_stream().cuda_stream
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 class _SceneData:
@@ -114,7 +119,7 @@ class Scene:
         B.epo_set_poses(self.handle, np.ascontiguousarray(T, dtype=np.float64).reshape(self.n_views, 12))
 
     def get_poses(self) -> np.ndarray:
-        T = np.zeros((self.n_views, 12))
+        T = np.empty((self.n_views, 12))
         B.epo_get_poses(self.handle, T)
         return T
 
@@ -132,8 +137,8 @@ class Scene:
 
     # ---- evaluation ----
     def loss_and_grad(self):
-        loss = np.zeros(self.n_scenes)
-        grad = np.zeros((self.n_views, 6))
+        loss = np.empty(self.n_scenes)
+        grad = np.empty((self.n_views, 6))
         B.epo_loss_and_grad(self.handle, loss, grad)
         return loss, grad
 
