@@ -19,7 +19,7 @@
 // FMA products) beside a bound on their error; a sample whose bound is too wide, or that has a
 // decision within it, takes the FP64 form (sample_exact).  The final gather is a warp per pose; it
 // was one block that scanned every pair for every pose.  24 views of 256x192, 192 pairs, 0.57 M
-// evaluations: 200 us for the call (edge kernel 104, gather 98) before, 33 us now.
+// evaluations: 200 us for the call (edge kernel 104, gather 98) before, 26 us now.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -249,11 +249,12 @@ __device__ __forceinline__ float warp_sums8(const float* v, int lane) {
 }
 
 // blockIdx.y = pair; the block walks the source view's tiles of kNaThreads records.  The launch
-// gives each pair as many blocks as make about kNaEdgeBlocks in all, so that a block's form is
-// built for more than one tile when the pairs alone fill the GPU.
-constexpr int kNaEdgeBlocks = 8 * 152;
+// gives each pair as many blocks as make one wave of four per SM in all: building a pair's form is a
+// chain of FP64 on one warp while the others wait, so a block does it for several tiles.  The call on
+// 24 views of 256x192: 26.4 us; two waves 30.3, four 36.6; at three blocks per SM (72 registers) 32.6.
+constexpr int kNaEdgeBlocks = 4 * 152;
 
-__global__ void __launch_bounds__(kNaThreads) k_na_edge(epo_noalloc_problem pb, NaScratch* S) {
+__global__ void __launch_bounds__(kNaThreads, 4) k_na_edge(epo_noalloc_problem pb, NaScratch* S) {
   __shared__ float s_red[2][kNaThreads / 32][kNaAcc];
   __shared__ NaForm s_f;
   __shared__ double s_Ki[4], s_Kj[4];
