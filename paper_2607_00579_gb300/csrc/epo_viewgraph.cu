@@ -11,7 +11,7 @@
 // that evaluation is ~200 instructions of the 1/64-rate FP64 pipe per grid pixel (24 views of
 // 518x392 at stride 4: 2.5 ms), so every grid pixel first runs in FP32 beside a bound on its error,
 // and only those with a decision inside the bound (well under 1 % of them) are kept in shared
-// memory and evaluated in FP64, 32 to a warp (the same 24 views: 2544 -> 146 us for the whole call).
+// memory and evaluated in FP64, 32 to a warp (the same 24 views: 2544 -> 131 us for the whole call).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -73,7 +73,7 @@ __device__ __noinline__ bool trip_exact(const VgView& vi, const VgView& vj, cons
 constexpr int kVgThreads = 256;
 constexpr int kVgRound = 1024;           // grid pixels between two looks at the kept ones
 constexpr int kVgExact = 2 * kVgRound;   // room for the kept ones: evaluated once half full
-constexpr int kVgBlocks = 5 * 152;  // one wave of resident blocks: fewer pairs are split over several
+constexpr int kVgBlocks = 4 * 152;  // one wave of resident blocks: fewer pairs are split over several
 
 // One direction of a pair in FP32: Y = M X + t, and the constants of the bound
 //   |Y_r - Y_r(FP64)| <= E = z Ca + Cb.
@@ -88,25 +88,26 @@ struct VgDir {
 };
 
 // Projects (X0, X1, z) with |Y_r| errors below E: q = Y_0,1 / Y_2 and the bound eq on its error.
-// Returns 1 in front (q, eq valid), 0 behind for certain, -1 not decided.  For e = E / Y2 <= 1/64,
-// |q - q*| <= e (1 + |q|) / (1 - e) plus 4u |q| for the reciprocal and the product.
-__device__ __forceinline__ int project(const VgDir& d, float X0, float X1, float z, float E, float& qu, float& qv,
-                                       float& eu, float& ev) {
+// front: in front for certain and q, eq valid; behind: behind for certain; neither: not decided (near
+// the camera plane, not a number, or where E could underflow).  For e = E / Y2 <= 1/64,
+// |q - q*| <= e (1 + |q|) / (1 - e) plus 4u |q| for the reciprocal and the product.  No branches: the
+// callers keep what the flags allow.
+__device__ __forceinline__ void project(const VgDir& d, float X0, float X1, float z, float E, float& qu, float& qv,
+                                        float& eu, float& ev, bool& front, bool& behind) {
   constexpr float u = epo::kU32;
   const float Y0 = fmaf(d.M[2], z, fmaf(d.M[1], X1, fmaf(d.M[0], X0, d.t[0])));
   const float Y1 = fmaf(d.M[5], z, fmaf(d.M[4], X1, fmaf(d.M[3], X0, d.t[1])));
   const float Y2 = fmaf(d.M[8], z, fmaf(d.M[7], X1, fmaf(d.M[6], X0, d.t[2])));
-  if (!(fabsf(Y2) > 1e-20f)) return -1;  // not a number, or where E could underflow
-  if (Y2 < -E) return 0;
   float iz;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(iz) : "f"(Y2));
   const float e = E * iz;
-  if (!(e >= 0.f && e <= 1.f / 64.f)) return -1;  // near the camera plane, or not a number
+  front = Y2 > 1e-20f && e <= 1.f / 64.f;
+  behind = Y2 < -1e-20f && Y2 < -E;
   qu = Y0 * iz;
   qv = Y1 * iz;
-  eu = fmaf(1.05f * e, 1.f + fabsf(qu), 4.f * u * fabsf(qu));
-  ev = fmaf(1.05f * e, 1.f + fabsf(qv), 4.f * u * fabsf(qv));
-  return 1;
+  const float e1 = 1.05f * e;
+  eu = fmaf(e1 + 4.f * u, fabsf(qu), e1);
+  ev = fmaf(e1 + 4.f * u, fabsf(qv), e1);
 }
 
 // Pixel coordinate f q + c and its error bound (the rounded f and c, the FMA, the comparisons).
@@ -116,8 +117,9 @@ __device__ __forceinline__ float pixel(float f, float c, float q, float eq, floa
   return p;
 }
 
-// Five blocks per SM (48 registers): 166 us for the call on 24 views; three 177, four 169, six 195.
-__global__ void __launch_bounds__(kVgThreads, 5) k_viewgraph(const VgView* views, const float* depth, int n, int stride,
+// Four blocks per SM (64 registers): 131 us for the call on 24 views; five 145. The trips run without
+// branches; with an early exit at every decision 146.
+__global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views, const float* depth, int n, int stride,
                                                           double tau, int per_block, uint2* counts) {
   constexpr float u = epo::kU32;
   __shared__ VgView vi, vj;
@@ -207,8 +209,8 @@ __global__ void __launch_bounds__(kVgThreads, 5) k_viewgraph(const VgView* views
   for (int round = g0; round < g1; round += kVgRound) {
     const int end = min(g1, round + kVgRound);
     for (int base = round; base < end; base += kStep) {
-      int known[ILP];  // 1 counted, 0 not, -1 an FP32 decision is in doubt, 2 not decided yet
       float z[ILP], qu[ILP], qv[ILP], eu[ILP], ev[ILP], zj[ILP], xf[ILP], yf[ILP];
+      bool doubt[ILP], on[ILP];  // an FP32 decision is in doubt; so far the trip holds
       int at[ILP];
 #pragma unroll
       for (int k = 0; k < ILP; ++k) {
@@ -226,43 +228,38 @@ __global__ void __launch_bounds__(kVgThreads, 5) k_viewgraph(const VgView* views
       }
 #pragma unroll
       for (int k = 0; k < ILP; ++k) {
-        known[k] = 0;
-        at[k] = -1;
-        if (!(z[k] > 0.f) || !isfinite(z[k])) continue;
-        ++valid;
-        known[k] = project(fwd, (xf[k] - cxi) * rfx * z[k], (yf[k] - cyi) * rfy * z[k], z[k], fmaf(z[k], fwd.Ca, fwd.Cb),
-                           qu[k], qv[k], eu[k], ev[k]);
-        if (known[k] != 1) continue;
+        const bool live = z[k] > 0.f && z[k] < INFINITY;
+        valid += live;
+        bool front, behind;
+        project(fwd, (xf[k] - cxi) * rfx * z[k], (yf[k] - cyi) * rfy * z[k], z[k], fmaf(z[k], fwd.Ca, fwd.Cb), qu[k], qv[k],
+                eu[k], ev[k], front, behind);
         float tu, tv;
         const float up = pixel(fxj, cxj, qu[k], eu[k], tu), vp = pixel(fyj, cyj, qv[k], ev[k], tv);
-        known[k] = up < -tu || up - Wm1 > tu || vp < -tv || vp - Hm1 > tv ? 0 : -1;  // outside view j, or perhaps
-        const float fu = floorf(up), fv = floorf(vp), ru = up - fu, rv = vp - fv;
-        if (up >= tu && Wm1 - up >= tu && vp >= tv && Hm1 - vp >= tv && fabsf(ru - 0.5f) > tu && fabsf(rv - 0.5f) > tv) {
-          known[k] = 2;
-          at[k] = ((int)fv + (rv > 0.5f)) * vj.W + (int)fu + (ru > 0.5f);
-        }
+        const float ou = up - Wm1, ov = vp - Hm1;
+        const bool outside = up < -tu || ou > tu || vp < -tv || ov > tv;
+        const float fu = floorf(up), fv = floorf(vp), ru = up - fu - 0.5f, rv = vp - fv - 0.5f;
+        on[k] = live && front && up >= tu && -ou >= tu && vp >= tv && -ov >= tv && fabsf(ru) > tu && fabsf(rv) > tv;
+        doubt[k] = live && !on[k] && !behind && !(front && outside);
+        at[k] = on[k] ? ((int)fv + (rv > 0.f)) * vj.W + (int)fu + (ru > 0.f) : 0;
       }
 #pragma unroll
-      for (int k = 0; k < ILP; ++k) zj[k] = at[k] >= 0 ? dj[at[k]] : 0.f;
+      for (int k = 0; k < ILP; ++k) zj[k] = on[k] ? dj[at[k]] : 0.f;
 #pragma unroll
       for (int k = 0; k < ILP; ++k) {
-        if (known[k] == 2) {
-          known[k] = 0;
-          if (zj[k] > 0.f && isfinite(zj[k])) {
-            const float E = fmaf(zj[k], fmaf(bwd.m, fmaxf(eu[k], ev[k]), bwd.Ca), bwd.Cb);
-            float bu, bv;
-            known[k] = project(bwd, qu[k] * zj[k], qv[k] * zj[k], zj[k], E, bu, bv, eu[k], ev[k]);
-            if (known[k] == 1) {
-              float tu, tv;
-              const float dx = pixel(fxi, cxi, bu, eu[k], tu) - xf[k], dy = pixel(fyi, cyi, bv, ev[k], tv) - yf[k];
-              const float d = sqrtf(fmaf(dx, dx, dy * dy));
-              const float td = tu + tv + 8.f * u * (d + tf);
-              known[k] = d + td < tf ? 1 : (d - td > tf ? 0 : -1);
-            }
-          }
-        }
-        good += known[k] == 1;
-        if (known[k] < 0) s_list[atomicAdd(&s_count, 1)] = base + k * kVgThreads + (int)threadIdx.x;
+        on[k] = zj[k] > 0.f && zj[k] < INFINITY;  // only trips that hold so far have read a depth
+        const float E = fmaf(zj[k], fmaf(bwd.m, fmaxf(eu[k], ev[k]), bwd.Ca), bwd.Cb);
+        float bu, bv;
+        bool front, behind;
+        project(bwd, qu[k] * zj[k], qv[k] * zj[k], zj[k], E, bu, bv, eu[k], ev[k], front, behind);
+        float tu, tv;
+        const float dx = pixel(fxi, cxi, bu, eu[k], tu) - xf[k], dy = pixel(fyi, cyi, bv, ev[k], tv) - yf[k];
+        float d;
+        asm("sqrt.approx.f32 %0, %1;" : "=f"(d) : "f"(fmaf(dx, dx, dy * dy)));  // relative error below 2^-22
+        const float td = tu + tv + 10.f * u * (d + tf);
+        const bool near = front && d + td < tf, far = front && d - td > tf;
+        good += on[k] && near;
+        doubt[k] = doubt[k] || (on[k] && !near && !far && !behind);
+        if (doubt[k]) s_list[atomicAdd(&s_count, 1)] = base + k * kVgThreads + (int)threadIdx.x;
       }
     }
     __syncthreads();
@@ -324,7 +321,7 @@ extern "C" epo_status epo_build_viewgraph(int32_t n_views, const int32_t* W, con
     uint2* d_counts = reinterpret_cast<uint2*>(d_buf + view_bytes);
     // one block per ordered pair; with few pairs each pair's grid is split over several blocks
     // (at least 512 pixels each) so that they fill the GPU, in one wave: each block forms its pair's
-    // constants in FP64 first (24 views: 146 us unsplit, 156 in halves, 168 in quarters)
+    // constants in FP64 first (24 views, with branches: 146 us unsplit, 156 in halves, 168 in quarters)
     int64_t grid = 1;
     for (int v = 0; v < n; ++v)
       grid = std::max(grid, (int64_t)((W[v] + stride - 1) / stride) * ((H[v] + stride - 1) / stride));
