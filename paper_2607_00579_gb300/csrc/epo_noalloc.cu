@@ -260,7 +260,9 @@ __global__ void __launch_bounds__(kNaThreads, 4) k_na_edge(epo_noalloc_problem p
   __shared__ double s_Ki[4], s_Kj[4];
   const int p = blockIdx.y;
   const int i = pb.pairs[2 * p], j = pb.pairs[2 * p + 1];
-  const int64_t r0 = pb.rec_off[i], n = pb.rec_off[i + 1] - r0;
+  // no more tiles than the caller's maximum of records per view makes
+  const int64_t most = (pb.max_records_per_view + kNaThreads - 1) / kNaThreads * kNaThreads;
+  const int64_t r0 = pb.rec_off[i], n = min(pb.rec_off[i + 1] - r0, most);
   const int W = pb.W[j], H = pb.H[j];
   const float* map = pb.maps + pb.map_off[j];
   epo::griddep_launch_dependents();

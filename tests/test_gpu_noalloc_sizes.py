@@ -60,3 +60,16 @@ def test_sizes(n, counts, pairs, spread, norm_mode):
     o = oracle.scene_from_synth(sc, [m.astype(np.float64) for m in maps]).loss_grad(
         sc.T_init, lam=10.0, norm_mode=oracle.NORM_ALL if norm_mode == B.EPO_NORM_ALL else oracle.NORM_VALID)
     check_against_oracle(got_loss, got_grad, o, sc.pairs, sc.T_init)
+
+
+def test_records_beyond_the_stated_maximum_are_left_out():
+    """The tiles that max_records_per_view makes bound the work: of a view with more records only those
+    of its first tiles (256 each) count."""
+    sc, maps = scene(3, [600, 300, 256], [(0, 1), (1, 2), (2, 0)])
+    run = Problem(sc, maps)
+    run.prob.max_records_per_view = 250
+    got_loss, got_grad = run(sc.T_init, B.EPO_NORM_VALID)
+    keep = np.concatenate([np.arange(sc.rec_off[v], sc.rec_off[v] + 256) for v in range(3)])
+    o = oracle.OracleScene(sc.W, sc.H, sc.K, np.arange(4, dtype=np.int64) * 256, sc.rec[keep],
+                           [m.astype(np.float64) for m in maps], sc.pairs).loss_grad(sc.T_init, lam=10.0)
+    check_against_oracle(got_loss, got_grad, o, sc.pairs, sc.T_init)
