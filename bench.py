@@ -594,7 +594,7 @@ ACC_STEPS = 100  # optimisation steps behind the final-accuracy comparisons
 
 def viewgraph_leg(epo, torch, wl, stride=4):
     """Viewgraph estimation (Section 3, Eq. 2): every ordered pair's round-trip fraction over
-    a grid of source pixels, on the GPU in FP64, at the initial poses and depths."""
+    a grid of source pixels, on the GPU, at the initial poses and depths."""
     sc = wl.scenes[0]
     depth = torch.cat([torch.from_numpy(d).reshape(-1) for d in sc.depth]).cuda()
     run = lambda: epo.build_viewgraph(sc.W, sc.H, sc.K, sc.T_init, depth, stride=stride, tau=3.0, min_frac=0.125)
@@ -610,7 +610,7 @@ def viewgraph_leg(epo, torch, wl, stride=4):
     return {"ms": ms, "round_trips": trips, "round_trips_per_s": trips / (ms * 1e-3), "grid_stride": stride,
             "tau_px": 3.0, "min_frac": 0.125, "pairs_kept": int(len(pairs)),
             "pairs_candidate": sc.n_views * (sc.n_views - 1),
-            "note": "wall time of epo_build_viewgraph (FP64 round trips, host copy of the fraction matrix)"}
+            "note": "wall time of epo_build_viewgraph (FP32 round trips, FP64 where a decision is in doubt, host copy of the counts)"}
 
 
 def refine_leg(epo, torch, wl, parts, dtypes, lr, evals, args, flush_l2, stream, sched):
@@ -684,9 +684,9 @@ def pose_mlp_leg(epo, torch, wl, parts, dtypes, lr, evals, args, flush_l2, strea
 
 
 def autograd_leg(epo, torch, s, T_init, evals, args, flush_l2, stream):
-    """Forward + adjoint through the autograd function at the current poses (two passes over
-    the samples: the adjoint recomputes every projection instead of storing per-sample
-    Jacobians), and the device memory this takes against a stored-Jacobian variant."""
+    """Forward + backward through the autograd function at the current poses (one fused pass that
+    keeps the poses' gradient instead of per-sample Jacobians), and the device memory this takes
+    against a stored-Jacobian variant."""
     s.set_poses(T_init)
     xi = torch.zeros((s.n_views, 6), dtype=torch.float64, device="cuda", requires_grad=True)
     for _ in range(3):
@@ -755,7 +755,7 @@ def plain_per_scene_leg(epo, torch, wl, s, parts, dtypes, lr, evals, args, flush
     rb, tb = pose_errors(Tb, wl.scenes)
     rp, tp = pose_errors(Tp, wl.scenes)
     return {"value": evals / (plain_ms * 1e-3), "unit": UNIT, "ms_per_step": plain_ms, "steps": n,
-            "schedule": "library default (block 256, 2 records per thread, plain loads), no autotuning",
+            "schedule": "library default (texture gather, block size and split from the amount of work), no autotuning",
             "speedup_of_batched_graph_step": None,
             "final_accuracy": {"steps": ACC_STEPS, "initial_rot_deg": r0, "initial_trans_frac": t0,
                                "batched_graph_rot_deg": rb, "batched_graph_trans_frac": tb,

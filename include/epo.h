@@ -414,7 +414,8 @@ epo_status epo_round_bf16(const float* src_dev, uint16_t* dst_dev, int64_t n, vo
  * (host): frac n_views x n_views (may be NULL; diagonal 0), pairs 2 x
  * n_views (n_views - 1) int32 capacity (may be NULL): the directed pairs of
  * the undirected pairs whose fraction is >= min_frac both ways, row-major;
- * *n_pairs their count.  FP64 on the device; synchronises.  Invalid sizes or
+ * *n_pairs their count.  The counts are those of an FP64 evaluation (pixels whose
+ * decisions an FP32 error bound settles are not evaluated twice); synchronises.  Invalid sizes or
  * intrinsics: EPO_ERR_INVALID_ARG; allocation failure: EPO_ERR_OOM. */
 epo_status epo_build_viewgraph(int32_t n_views, const int32_t* W, const int32_t* H, const double* K, const double* T,
                                const float* depth_dev, int32_t stride, double tau, double min_frac, double* frac,
