@@ -191,9 +191,11 @@ def _ptr(x):
         return ctypes.c_void_p(x)
     if hasattr(x, "data_ptr"):
         return ctypes.c_void_p(x.data_ptr())
-    if hasattr(x, "__array_interface__"):
+    if hasattr(type(x), "ctypes") and hasattr(x, "__array_interface__"):  # an array, without its ctypes object
         return ctypes.c_void_p(x.__array_interface__["data"][0])
-    raise TypeError(type(x))
+    if hasattr(x, "ctypes"):
+        return ctypes.c_void_p(x.ctypes.data)
+    raise TypeError(type(x))  # numpy scalars too: their interface names a temporary
 
 
 def epo_abi_version() -> int:
