@@ -173,8 +173,9 @@ class EdgeLoss:
     J_l(xi)^T of it: one pass over the samples instead of a forward and a recomputing adjoint
     (forward and backward, 200 views with 5.7e7 evaluations 895 -> 336 us, 120 views 400 -> 291; below
     that torch's own ~300 us per pass on the host is the limit, 48 views 301 -> 287).
-    Without a gradient, and in refinement scenes (whose fused pass also stores every sample's
-    derivative), the forward pass forms the loss only and the backward recomputes."""
+    Without a gradient, in refinement scenes (whose fused pass also stores every sample's
+    derivative), and where torch's current stream is not the scene's, the forward pass forms the loss
+    only and the backward recomputes."""
 
     _fn = None
 
@@ -210,7 +211,11 @@ class EdgeLoss:
                     return out, None, None
 
             cls._fn = _F
-        return cls._fn.apply(xi, scene, torch.is_grad_enabled() and xi.requires_grad and not getattr(scene, "refine", True))
+        # the kept gradient is torch's memory and the library's kernels run on the scene's stream: on
+        # another stream it could be handed out again before the backward has read it
+        fused = (torch.is_grad_enabled() and xi.requires_grad and not getattr(scene, "refine", True)
+                 and scene._stream == _current_stream())
+        return cls._fn.apply(xi, scene, fused)
 
 
 def distance_field(edges, stream: Optional[int] = None):

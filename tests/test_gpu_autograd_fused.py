@@ -63,3 +63,23 @@ def test_left_jacobian_and_twists_match_the_oracle():
     want = np.stack([2.0 * oracle.se3_left_jacobian(x[v]).T @ g[v] for v in range(40)])
     # the closed form of the oracle loses digits to cancellation at small angles
     assert np.abs(out.cpu().numpy() - want).max() < 1e-9
+
+
+def test_another_stream_keeps_no_buffer():
+    """The kept gradient is torch's memory, so a pass on another stream than the scene's keeps none."""
+    s = scene(60, 44, 20, 300, 4, False)
+    x = torch.full((20, 6), 0.01, dtype=torch.float64, device="cuda", requires_grad=True)
+    side = torch.cuda.Stream()
+    out = []
+    for st in (torch.cuda.current_stream(), side):
+        torch.cuda.synchronize()
+        with torch.cuda.stream(st):
+            L = epo.EdgeLoss.apply(x, s)
+            torch.cuda.synchronize()
+            kept = len(L.grad_fn.saved_tensors)
+            g = torch.autograd.grad(L.sum(), x)[0]
+            torch.cuda.synchronize()
+        out.append((kept, L.detach(), g))
+    assert [k for k, _, _ in out] == [2, 1]
+    assert torch.allclose(out[0][1], out[1][1], rtol=1e-13, atol=0)
+    assert (out[0][2] - out[1][2]).abs().max() <= 1e-12 * out[0][2].abs().max()
