@@ -179,8 +179,10 @@ __global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views
       m = fmaxf(m, fabsf(d.M[3 * r]) + fabsf(d.M[3 * r + 1]) + fabsf(d.M[3 * r + 2]));
     }
     const float mm = 1e-14f * nt[0] * nf[1];  // rows of |R_to| times columns of |R_from|
+    // the limits of either image hold for both directions: a trip indexes the depths of the other view
+    const float G = nt[3] < INFINITY ? nf[3] : INFINITY;
     d.m = 1.01f * m;
-    d.Ca = 1.01f * nf[3] * (10.f * u * m + mm);
+    d.Ca = 1.01f * G * (10.f * u * m + mm);
     d.Cb = 1.01f * (10.f * u * tm + mm * nf[2] + 1e-14f * nt[2]);
   }
   __syncthreads();

@@ -75,3 +75,44 @@ def test_viewgraph_counts_are_exact_where_decisions_are_close(n, W, H, stride, t
     want = oracle.viewgraph(np.full(n, W), np.full(n, H), K, T.reshape(n, 12), depths, stride=stride, tau=tau)
     assert np.array_equal(frac, want)
     assert np.array_equal(pairs, oracle.viewgraph_pairs(want, 0.125))
+
+
+def small_motion(r, n):
+    T = np.zeros((n, 3, 4))
+    for v in range(n):
+        T[v, :, :3] = synth._rotvec_to_matrix(r.normal(0, 0.03, 3))
+        T[v, :, 3] = r.normal(0, 0.2, 3)
+    return T.reshape(n, 12)
+
+
+@pytest.mark.parametrize("stride", [1, 3])
+def test_views_of_different_sizes(stride):
+    """Grids, borders and row pitches of each pair's own two views; 7 views, so that the pairs' grids
+    are split over several blocks by the largest one."""
+    r = np.random.default_rng(stride)
+    W, H = np.array([61, 200, 17, 96, 33, 128, 5]), np.array([47, 31, 90, 96, 150, 12, 4])
+    K = np.stack([1.1 * W, 1.2 * H, W / 2 - 0.3, H / 2 + 0.4], axis=1)
+    T = small_motion(r, len(W))
+    depths = [r.uniform(3, 5, (h, w)).astype(np.float32) for w, h in zip(W, H)]
+    frac, _ = epo.build_viewgraph(W, H, K, T, [torch.from_numpy(d).cuda() for d in depths], stride=stride, tau=3.0)
+    assert np.array_equal(frac, oracle.viewgraph(W, H, K, T, depths, stride=stride, tau=3.0))
+    assert len(np.unique(frac)) > 20
+
+
+def test_target_beyond_32_bit_pixel_indices():
+    """A small view against one of 65536x40000 pixels, whose lower rows an int does not number.  Same
+    pose, constant depth, powers of two throughout: pixel (x, y) of the one is (128 x, 128 y) of the
+    other and every trip returns to its own pixel, except where the huge view's depth is cleared."""
+    W, H = np.array([512, 65536]), np.array([313, 40000])
+    K = np.array([[512, 256, 256, 160], [65536, 32768, 32768, 20480]], dtype=np.float64)
+    depth = torch.full((512 * 313 + 65536 * 40000,), 4.0, device="cuda")
+    depth[512 * 313:].view(40000, 65536)[36000:38000] = 0.0
+    frac, _ = epo.build_viewgraph(W, H, K, np.tile(np.eye(3, 4).reshape(-1), (2, 1)), depth, stride=5, tau=0.75)
+    del depth
+    torch.cuda.empty_cache()
+    cleared = lambda y: (y >= 36000) & (y < 38000)
+    y = 128 * np.arange(0, 313, 5)
+    assert frac[0, 1] == np.sum(~cleared(y)) / len(y)
+    x, y = np.arange(0, 65536, 5), np.arange(0, 40000, 5)
+    y = y[~cleared(y)]
+    assert frac[1, 0] == int(np.sum(x <= 128 * 511)) * int(np.sum(y <= 128 * 312)) / (len(x) * len(y))
