@@ -89,7 +89,8 @@ struct VgDir {
 
 // Projects (X0, X1, z) with |Y_r| errors below E: q = Y_0,1 / Y_2 and the bound eq on its error.
 // front: in front for certain and q, eq valid; behind: behind for certain; neither: not decided (near
-// the camera plane, not a number, or where E could underflow).  For e = E / Y2 <= 1/64,
+// the camera plane, not a number, where E could underflow, or from 1e30 on: the reciprocal is flushed
+// to zero above 2^126 and a sum that overflowed has lost its sign).  For e = E / Y2 <= 1/64,
 // |q - q*| <= e (1 + |q|) / (1 - e) plus 4u |q| for the reciprocal and the product.  No branches: the
 // callers keep what the flags allow.
 __device__ __forceinline__ void project(const VgDir& d, float X0, float X1, float z, float E, float& qu, float& qv,
@@ -101,8 +102,8 @@ __device__ __forceinline__ void project(const VgDir& d, float X0, float X1, floa
   float iz;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(iz) : "f"(Y2));
   const float e = E * iz;
-  front = Y2 > 1e-20f && e <= 1.f / 64.f;
-  behind = Y2 < -1e-20f && Y2 < -E;
+  front = Y2 > 1e-20f && Y2 < 1e30f && e <= 1.f / 64.f;
+  behind = Y2 < -1e-20f && Y2 > -1e30f && Y2 < -E;
   qu = Y0 * iz;
   qv = Y1 * iz;
   const float e1 = 1.05f * e;

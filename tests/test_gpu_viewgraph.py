@@ -116,3 +116,25 @@ def test_target_beyond_32_bit_pixel_indices():
     x, y = np.arange(0, 65536, 5), np.arange(0, 40000, 5)
     y = y[~cleared(y)]
     assert frac[1, 0] == int(np.sum(x <= 128 * 511)) * int(np.sum(y <= 128 * 312)) / (len(x) * len(y))
+
+
+@pytest.mark.parametrize("far", [8e37, 9e37, 2e38, 3.4028234663852886e38])
+@pytest.mark.parametrize("where", ["source", "both"])
+def test_depths_near_the_largest_float(far, where):
+    """Depths at which a reciprocal in FP32 is subnormal or zero (FLT_MAX marks the sky in some depth
+    maps): every trip through them is decided in FP64."""
+    r = np.random.default_rng(4)
+    n, W, H = 4, 63, 47
+    K = np.tile([70.0, 70.0, 30.3, 22.8], (n, 1))
+    T = small_motion(r, n)
+    T[1] = T[0]  # two views of one orientation, shifted
+    T[1, 3] += 0.2
+    depths = [r.uniform(3, 5, (H, W)).astype(np.float32) for _ in range(n)]
+    for v, d in enumerate(depths):
+        if where == "both" or v % 2 == 0:
+            d[:30] = np.float32(far)
+    frac, _ = epo.build_viewgraph(np.full(n, W), np.full(n, H), K, T, [torch.from_numpy(d).cuda() for d in depths],
+                                  stride=1, tau=3.0)
+    want = oracle.viewgraph(np.full(n, W), np.full(n, H), K, T, depths, stride=1, tau=3.0)
+    assert np.array_equal(frac, want)
+    assert where == "source" or want[0, 1] > 0.9
