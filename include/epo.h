@@ -416,7 +416,8 @@ epo_status epo_round_bf16(const float* src_dev, uint16_t* dst_dev, int64_t n, vo
  * the undirected pairs whose fraction is >= min_frac both ways, row-major;
  * *n_pairs their count.  The counts are those of an FP64 evaluation (pixels whose
  * decisions an FP32 error bound settles are not evaluated twice); synchronises.  Invalid sizes or
- * intrinsics: EPO_ERR_INVALID_ARG; allocation failure: EPO_ERR_OOM. */
+ * intrinsics: EPO_ERR_INVALID_ARG; a view with more than 2^32 - 1 grid pixels:
+ * EPO_ERR_TOO_LARGE; allocation failure: EPO_ERR_OOM. */
 epo_status epo_build_viewgraph(int32_t n_views, const int32_t* W, const int32_t* H, const double* K, const double* T,
                                const float* depth_dev, int32_t stride, double tau, double min_frac, double* frac,
                                int32_t* pairs, int32_t* n_pairs, void* cuda_stream);

@@ -74,6 +74,7 @@ constexpr int kVgThreads = 256;
 constexpr int kVgRound = 1024;           // grid pixels between two looks at the kept ones
 constexpr int kVgExact = 2 * kVgRound;   // room for the kept ones: evaluated once half full
 constexpr int kVgBlocks = 4 * 152;  // one wave of resident blocks: fewer pairs are split over several
+constexpr int64_t kVgMaxCount = 1 << 30;  // grid pixels of a block: its loop counts in int
 
 // One direction of a pair in FP32: Y = M X + t, and the constants of the bound
 //   |Y_r - Y_r(FP64)| <= E = z Ca + Cb.
@@ -187,8 +188,11 @@ __global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views
     d.Cb = 1.01f * (10.f * u * tm + mm * nf[2] + 1e-14f * nt[2]);
   }
   __syncthreads();
-  const int gw = (vi.W + stride - 1) / stride, gh = (vi.H + stride - 1) / stride;
-  const int g0 = blockIdx.y * per_block, g1 = min(gw * gh, g0 + per_block);
+  // the block's grid pixels are first .. first + count - 1 of the view's, which an int may not number,
+  // and have numbers of their own from 0
+  const unsigned gw = (unsigned)((vi.W - 1) / stride + 1), gh = (unsigned)((vi.H - 1) / stride + 1);
+  const int64_t first = (int64_t)blockIdx.y * per_block;
+  const int count = (int)max((int64_t)0, min((int64_t)per_block, (int64_t)gw * gh - first));  // 0: a smaller view's grid
   const float fxi = (float)vi.K[0], fyi = (float)vi.K[1], cxi = (float)vi.K[2], cyi = (float)vi.K[3];
   const float fxj = (float)vj.K[0], fyj = (float)vj.K[1], cxj = (float)vj.K[2], cyj = (float)vj.K[3];
   const float rfx = (float)(1.0 / vi.K[0]), rfy = (float)(1.0 / vi.K[1]);
@@ -201,23 +205,24 @@ __global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views
   // 518x392, two: 166)
   constexpr int ILP = 2;
   constexpr int kStep = ILP * kVgThreads;
-  const int dr = kStep / gw, dc = kStep % gw;
-  int row[ILP], col[ILP];
+  const unsigned dr = kStep / gw, dc = kStep % gw;
+  const unsigned row0 = (unsigned)(first / gw), col0 = (unsigned)(first % gw);
+  unsigned row[ILP], col[ILP];
 #pragma unroll
   for (int k = 0; k < ILP; ++k) {
-    const int g = g0 + k * kVgThreads + (int)threadIdx.x;
-    row[k] = g / gw;
+    const unsigned g = col0 + k * kVgThreads + threadIdx.x;
+    row[k] = row0 + g / gw;
     col[k] = g % gw;
   }
-  for (int round = g0; round < g1; round += kVgRound) {
-    const int end = min(g1, round + kVgRound);
+  for (int round = 0; round < count; round += kVgRound) {
+    const int end = min(count, round + kVgRound);
     for (int base = round; base < end; base += kStep) {
       float z[ILP], qu[ILP], qv[ILP], eu[ILP], ev[ILP], zj[ILP], xf[ILP], yf[ILP];
       bool doubt[ILP], on[ILP];  // an FP32 decision is in doubt; so far the trip holds
       int at[ILP];
 #pragma unroll
       for (int k = 0; k < ILP; ++k) {
-        const int x = col[k] * stride, y = row[k] * stride;
+        const int x = (int)col[k] * stride, y = (int)row[k] * stride;
         const bool in = base + k * kVgThreads + (int)threadIdx.x < end;
         z[k] = in ? di[(int64_t)y * vi.W + x] : 0.f;
         xf[k] = (float)x;
@@ -268,9 +273,10 @@ __global__ void __launch_bounds__(kVgThreads, 4) k_viewgraph(const VgView* views
     __syncthreads();
     const int kept = s_count;
     __syncthreads();  // every thread has read it before the next round appends
-    if (kept > kVgExact - kVgRound || end == g1) {
+    if (kept > kVgExact - kVgRound || end == count) {
       for (int k = threadIdx.x; k < kept; k += kVgThreads) {
-        const int x = s_list[k] % gw * stride, y = s_list[k] / gw * stride;
+        const int64_t g = first + s_list[k];
+        const int x = (int)(g % gw) * stride, y = (int)(g / gw) * stride;
         good += trip_exact(vi, vj, depth, x, y, di[(int64_t)y * vi.W + x], tau);
       }
       __syncthreads();
@@ -299,7 +305,7 @@ extern "C" epo_status epo_build_viewgraph(int32_t n_views, const int32_t* W, con
     return EPO_ERR_INVALID_ARG;
   const int n = n_views;
   std::vector<VgView> hv(n);
-  int64_t off = 0;
+  int64_t off = 0, grid = 1;  // grid: the most grid pixels of a view
   for (int v = 0; v < n; ++v) {
     if (W[v] < 1 || H[v] < 1) return EPO_ERR_INVALID_ARG;
     hv[v].W = W[v];
@@ -309,7 +315,9 @@ extern "C" epo_status epo_build_viewgraph(int32_t n_views, const int32_t* W, con
     for (int k = 0; k < 4; ++k) hv[v].K[k] = K[4 * v + k];
     for (int k = 0; k < 12; ++k) hv[v].T[k] = T[12 * v + k];
     if (!(hv[v].K[0] > 0) || !(hv[v].K[1] > 0)) return EPO_ERR_INVALID_ARG;
+    grid = std::max(grid, (int64_t)((W[v] - 1) / stride + 1) * ((H[v] - 1) / stride + 1));
   }
+  if (grid > (int64_t)UINT32_MAX) return EPO_ERR_TOO_LARGE;  // the counts are 32-bit
   cudaStream_t st = (cudaStream_t)cuda_stream;
   // the view table and the pairs' counts in one allocation
   const size_t view_bytes = sizeof(VgView) * n, count_bytes = sizeof(uint2) * (size_t)n * n;
@@ -325,11 +333,9 @@ extern "C" epo_status epo_build_viewgraph(int32_t n_views, const int32_t* W, con
     // one block per ordered pair; with few pairs each pair's grid is split over several blocks
     // (at least 512 pixels each) so that they fill the GPU, in one wave: each block forms its pair's
     // constants in FP64 first (24 views, with branches: 146 us unsplit, 156 in halves, 168 in quarters)
-    int64_t grid = 1;
-    for (int v = 0; v < n; ++v)
-      grid = std::max(grid, (int64_t)((W[v] + stride - 1) / stride) * ((H[v] + stride - 1) / stride));
     const int64_t pairs_n = (int64_t)n * (n - 1);
-    const int64_t split = std::min<int64_t>(std::max<int64_t>(1, kVgBlocks / std::max<int64_t>(pairs_n, 1)), (grid + 511) / 512);
+    int64_t split = std::min<int64_t>(std::max<int64_t>(1, kVgBlocks / std::max<int64_t>(pairs_n, 1)), (grid + 511) / 512);
+    split = std::max(split, (grid + kVgMaxCount - 1) / kVgMaxCount);
     const int per_block = (int)((grid + split - 1) / split);
     if (cudaMemcpyAsync(d_buf, hv.data(), view_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemsetAsync(d_counts, 0, count_bytes, st) != cudaSuccess)

@@ -138,3 +138,31 @@ def test_depths_near_the_largest_float(far, where):
     want = oracle.viewgraph(np.full(n, W), np.full(n, H), K, T, depths, stride=1, tau=3.0)
     assert np.array_equal(frac, want)
     assert where == "source" or want[0, 1] > 0.9
+
+
+@pytest.mark.parametrize("W1,H1", [(49981, 42966), (50000, 50000)])  # 2^31 - 2 pixels, and beyond an int
+def test_grids_at_and_beyond_32_bit_numbers(W1, H1):
+    """Every pixel of a huge view against a small one: as above, with a few rows of valid depths."""
+    W, H = np.array([W1, (W1 - 1) // 128 + 1]), np.array([H1, (H1 - 1) // 128 + 1])
+    K = np.array([[65536, 65536, 32768, 32768], [512, 512, 256, 256]], dtype=np.float64)
+    depth = torch.zeros(W1 * H1 + int(W[1]) * int(H[1]), device="cuda")
+    depth[W1 * H1:] = 4.0
+    rows = np.array([0, 1, 128, 128 * 200 - 1, 128 * 200, 128 * 300, H1 - 1])
+    for y in rows:
+        depth[W1 * y:W1 * (y + 1)] = 4.0
+    frac, _ = epo.build_viewgraph(W, H, K, np.tile(np.eye(3, 4).reshape(-1), (2, 1)), depth, stride=1, tau=0.75)
+    del depth
+    torch.cuda.empty_cache()
+    inside = int(np.sum(np.arange(W1) <= 128 * (W[1] - 1))) * int(np.sum(rows <= 128 * (H[1] - 1)))
+    assert frac[0, 1] == inside / (W1 * len(rows))
+    back = np.isin(128 * np.arange(H[1]), rows).sum()
+    assert frac[1, 0] == int(back) / int(H[1])
+
+
+def test_stride_beyond_the_image_and_too_many_grid_pixels():
+    d = torch.full((2 * 40 * 30,), 4.0, device="cuda")
+    K, T = np.tile([64.0, 64.0, 20.0, 15.0], (2, 1)), np.tile(np.eye(3, 4).reshape(-1), (2, 1))
+    frac, _ = epo.build_viewgraph([40, 40], [30, 30], K, T, d, stride=2**31 - 1, tau=3.0)
+    assert np.array_equal(frac, [[0, 1], [1, 0]])
+    with pytest.raises(epo.EpoError):  # refused on the host, before the depths are touched
+        epo.build_viewgraph([2**17, 40], [2**16, 30], K, T, d, stride=1, tau=3.0)
