@@ -309,8 +309,8 @@ epo_status epo_last_loss(epo_scene_t scene, double* loss);
 /* Samples of the most recent evaluation whose FP32 position lay within its
  * rounding-error bound of a discontinuity (bilinear cell line, image border,
  * depth threshold, clamp) and were re-evaluated with FP64 decisions
- * (queued), and those that found their block's buffer full and kept their
- * FP32 decisions (overflow, normally 0).  Synchronises. */
+ * (queued).  overflow, those left with FP32 decisions, is 0: there are
+ * none.  Synchronises. */
 epo_status epo_fixup_stats(epo_scene_t scene, int64_t* queued, int64_t* overflow);
 
 /* Device time in milliseconds of the edge kernel (lift, projection, sampling,

@@ -57,6 +57,9 @@ struct Sched {
   int halves = 1;  // 2: the block does the work item of one twice as wide (k_edge_pose, HALVES)
   int block = 256;
   int tail = 0;    // pairs per work item of the last wave (0 = not split)
+  bool operator==(const Sched& o) const {
+    return gather == o.gather && rpt == o.rpt && halves == o.halves && block == o.block && tail == o.tail;
+  }
 };
 
 }  // namespace
@@ -110,7 +113,10 @@ struct epo_scene {
   double *d_pp64 = nullptr, *d_K64 = nullptr, *d_pair_acc = nullptr, *d_grad = nullptr,
          *d_loss = nullptr, *d_m = nullptr, *d_v = nullptr, *d_bpow = nullptr, *d_lambda = nullptr,
          *d_T = nullptr, *d_T_eval = nullptr;
-  unsigned int *d_qcount = nullptr, *d_qoverflow = nullptr;
+  unsigned int* d_qcount = nullptr;
+  unsigned int* d_left_bits = nullptr;  // EdgeArgs::left_bits, left_words of them
+  size_t left_words = 0;
+  Sched left_for{0, 0, 0, 0, 0};  // the schedule they were last sized for
   int* d_tile_counter = nullptr;
   int max_pairs = 1;
   int64_t* d_step = nullptr;
@@ -439,6 +445,8 @@ StepArgs step_args(epo_scene* S, const double* T_eval, const double* gscale) {
 }
 
 int resident_blocks(epo_scene* S, const Sched& sc);
+int item_pairs(epo_scene* S, const Sched& sc);
+int grid_for(epo_scene* S, const Sched& sc);
 
 // Work items of the edge kernel, in the order the blocks claim them: (view, records
 // [begin, begin + n), pairs [q0, q1) of the view's outgoing pair list).  Each item covers
@@ -501,8 +509,20 @@ epo_status build_tiles(epo_scene* S, int tile, int tail, int grid) {
 // per resident block (items of at most `tail` pairs), with tail < 0 every item covers at most
 // -tail pairs (more, smaller items).
 epo_status build_tiles(epo_scene* S, const Sched& sc) {
-  if (sc.tail < 0) return build_tiles(S, sc.block * sc.rpt, -sc.tail, INT_MAX);
-  return build_tiles(S, sc.block * sc.rpt, sc.tail, sc.tail ? resident_blocks(S, sc) : 0);
+  epo_status st = sc.tail < 0 ? build_tiles(S, sc.block * sc.rpt, -sc.tail, INT_MAX)
+                              : build_tiles(S, sc.block * sc.rpt, sc.tail, sc.tail ? resident_blocks(S, sc) : 0);
+  if (st != EPO_OK || S->left_for == sc) return st;
+  // a bit for every sample of a block's work item: 87 KB per pair of the longest item for the default
+  // schedules on 152 SMs
+  const size_t words = (size_t)grid_for(S, sc) * item_pairs(S, sc) * (sc.block * sc.rpt / 32);
+  if (words > S->left_words) {  // graphs captured with smaller schedules keep theirs until the scene goes
+    ALLOC(S->d_left_bits, words);
+    CK(cudaMemsetAsync(S->d_left_bits, 0, words * 4, S->stream));
+    S->left_words = words;
+    S->graph_dirty = true;
+  }
+  S->left_for = sc;
+  return EPO_OK;
 }
 
 // The work items of the current schedule.
@@ -524,7 +544,7 @@ EdgeArgs edge_args(epo_scene* S) {
   a.pp = S->d_pp;
   a.pp64 = S->d_pp64;
   a.q_count = S->d_qcount;
-  a.q_overflow = S->d_qoverflow;
+  a.left_bits = S->d_left_bits;
   a.tile_counter = S->d_tile_counter;
   a.pair_active = S->d_active;
   a.tex = S->d_tex;
@@ -1005,11 +1025,8 @@ epo_status create_impl(int32_t n_scenes, const epo_scene_desc* descs, const epo_
     ALLOC(S->d_m, (size_t)6 * nv);
     ALLOC(S->d_v, (size_t)6 * nv);
     ALLOC(S->d_bpow, 2);
-    {
-      ALLOC(S->d_qcount, 1);
-      ALLOC(S->d_qoverflow, 1);
-      ALLOC(S->d_tile_counter, 1);
-    }
+    ALLOC(S->d_qcount, 1);
+    ALLOC(S->d_tile_counter, 1);
     ALLOC(S->d_lambda, 1);
     ALLOC(S->d_T_eval, (size_t)12 * nv);
     ALLOC(S->d_step, 1);
@@ -1179,7 +1196,6 @@ epo_status create_impl(int32_t n_scenes, const epo_scene_desc* descs, const epo_
     if (S->d_lift)
       CK(launch_lift_records(S->d_rec, S->rec_dtype, S->d_views, S->d_K64, (int)nv, (float)o.eps_z, S->d_lift, st));
     CK(cudaMemsetAsync(S->d_qcount, 0, 4, st));
-    CK(cudaMemsetAsync(S->d_qoverflow, 0, 4, st));
     CK(cudaMemsetAsync(S->d_step, 0, 8, st));
     CK(cudaMemsetAsync(S->d_flag, 0, 4, st));
     ALLOC(S->d_dbg, 4);
@@ -1760,12 +1776,11 @@ epo_status epo_set_wait_limit(epo_scene_t S, double seconds) {
 epo_status epo_fixup_stats(epo_scene_t S, int64_t* queued, int64_t* overflow) {
   EPO_RANGE("epo_fixup_stats");
   if (!S) return fail(S, EPO_ERR_INVALID_ARG, "null scene");
-  unsigned int h[2] = {0u, 0u};
-  CK(cudaMemcpyAsync(&h[0], S->d_qcount, 4, cudaMemcpyDeviceToHost, S->stream));
-  CK(cudaMemcpyAsync(&h[1], S->d_qoverflow, 4, cudaMemcpyDeviceToHost, S->stream));
+  unsigned int h = 0u;
+  CK(cudaMemcpyAsync(&h, S->d_qcount, 4, cudaMemcpyDeviceToHost, S->stream));
   CK(cudaStreamSynchronize(S->stream));
-  if (queued) *queued = h[0];
-  if (overflow) *overflow = h[1];
+  if (queued) *queued = h;
+  if (overflow) *overflow = 0;
   return EPO_OK;
 }
 

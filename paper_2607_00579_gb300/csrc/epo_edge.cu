@@ -135,10 +135,11 @@ constexpr int kAmbRun = 64;
 //   * the bilinear value and slopes are formed in FP32 from the cell fractions; the clamp
 //     decision d <= lambda takes the FP32 value unless it lies within its error bound of
 //     lambda, in which case the fractions and d are formed again in FP64.
-// Adds straight to the pair's FP64 accumulators.
+// add(slot, value): where the sample's terms of the pair's sums go.
 // rec: the sample's record (refine scenes reload its pixel and prior depth for an FP64 z).
-template <int MODE, int REC, int MAP, int REF>
-__device__ void exact_eval(const EdgeArgs& a, const AmbEntry& en, int64_t rec, double lam, float lamf) {
+template <int MODE, int REC, int MAP, int REF, class Add>
+__device__ __forceinline__ void exact_eval(const EdgeArgs& a, const AmbEntry& en, int64_t rec, double lam, float lamf,
+                                           const Add& add) {
   const int p = en.p;
   const PairParam& P = a.pp[en.q];
   // the pair's projective form from the pair setup: (Y3 u', Y3 v', Y3) = z B (u, v, 1) + c
@@ -191,10 +192,9 @@ __device__ void exact_eval(const EdgeArgs& a, const AmbEntry& en, int64_t rec, d
   const float dh = pass ? df : lamf;
   const float adh = fabsf(dh);
   const float rho = adh <= delta ? 0.5f * dh * dh : delta * (adh - 0.5f * delta);
-  double* acc = a.pair_acc + (size_t)kAcc * p;
   if constexpr (MODE != MODE_BWD) {
-    atomicAdd(acc + 0, (double)rho);
-    atomicAdd(acc + 1, 1.0);
+    add(0, rho);
+    add(1, 1.f);
   }
   if constexpr (MODE != MODE_FWD) {
     const float drho = pass ? (fabsf(df) <= delta ? df : copysignf(delta, df)) : 0.f;
@@ -203,12 +203,12 @@ __device__ void exact_eval(const EdgeArgs& a, const AmbEntry& en, int64_t rec, d
       const float xn = ((float)su * rz - P.cx) / P.fx, yn = ((float)sv * rz - P.cy) / P.fy;
       const float ga = drho * (P.fx * ddu), gb = drho * (P.fy * ddv), gc = -fmaf(ga, xn, gb * yn);
       const float gx = ga * rz, gy = gb * rz, gz = gc * rz;
-      atomicAdd(acc + 2, (double)gx);
-      atomicAdd(acc + 3, (double)gy);
-      atomicAdd(acc + 4, (double)gz);
-      atomicAdd(acc + 5, (double)fmaf(yn, gc, -gb));
-      atomicAdd(acc + 6, (double)fmaf(-xn, gc, ga));
-      atomicAdd(acc + 7, (double)fmaf(xn, gb, -(yn * ga)));
+      add(2, gx);
+      add(3, gy);
+      add(4, gz);
+      add(5, fmaf(yn, gc, -gb));
+      add(6, fmaf(-xn, gc, ga));
+      add(7, fmaf(xn, gb, -(yn * ga)));
       if constexpr (REF) {
         // R (x~, y~, 1) = dY/dz; dRho/dz = g . dY/dz; the focal terms as in the fast path (the
         // entry holds the record's unit-depth ray (x~, y~))
@@ -217,10 +217,76 @@ __device__ void exact_eval(const EdgeArgs& a, const AmbEntry& en, int64_t rec, d
         const float dz = gx * fmaf(r[0], xtf, fmaf(r[1], ytf, r[2])) + gy * fmaf(r[3], xtf, fmaf(r[4], ytf, r[5])) +
                          gz * fmaf(r[6], xtf, fmaf(r[7], ytf, r[8]));
         const float gr2 = gx * r[2] + gy * r[5] + gz * r[8];
-        atomicAdd(a.pair_facc + 2 * (size_t)p, (double)(zf * (gr2 - dz)));
-        atomicAdd(a.pair_facc + 2 * (size_t)p + 1, (double)(-gc));  // gx Y0 + gy Y1
+        add(8, zf * (gr2 - dz));
+        add(9, -gc);  // gx Y0 + gy Y1
         if constexpr (MODE == MODE_FUSED) a.dzr[P.dbase + rec] = dz;  // the fast path wrote 0
       }
+    }
+  }
+}
+
+// Straight to the FP64 accumulators of the entry's pair.
+template <int MODE, int REC, int MAP, int REF>
+__device__ __forceinline__ void exact_eval(const EdgeArgs& a, const AmbEntry& en, int64_t rec, double lam, float lamf) {
+  double* acc = a.pair_acc + (size_t)kAcc * en.p;
+  double* facc = REF ? a.pair_facc + 2 * (size_t)en.p : nullptr;
+  exact_eval<MODE, REC, MAP, REF>(a, en, rec, lam, lamf, [&](int slot, float x) {
+    atomicAdd(slot < kAcc ? acc + slot : facc + slot - kAcc, (double)x);
+  });
+}
+
+// Samples that find the block's buffer full (scenes whose views lie on each other's pixels: a step
+// from identical poses queues every sample) leave a bit each in the block's part of a.left_bits, a
+// word per 32 records of the item and pair, and follow the buffered ones once the item is done.  So
+// no sample keeps a decision that its bound does not settle, and which ones the buffer took, a
+// matter of timing, shows in the order of FP64 additions only.
+// mask: a warp's candidates; the first `fit` of them have a place in the buffer.
+__device__ __forceinline__ void leave_bits(const EdgeArgs& a, int words, int pair, int word, unsigned mask, int fit,
+                                           int lane) {
+  const bool left = (mask >> lane & 1u) && __popc(mask & ((1u << lane) - 1u)) >= fit;
+  const unsigned bits = __ballot_sync(0xffffffffu, left);
+  if (lane == 0) a.left_bits[((size_t)blockIdx.x * a.max_pairs + pair) * words + word] = bits;
+}
+
+// The exact path for the samples left in the block's bits for work item td, which are cleared.
+// entry(q, p, li): the AmbEntry of pair p's (PairParam q's) sample at record li of the item.  A word's
+// samples belong to one pair: a warp sums their terms (FP64, fixed order) and adds each sum once.  An
+// evaluation of 32 views of 518x392 at identical poses, all 5.2e6 samples in FP64: 1004 us (one addition
+// per sample and term 2168; with FP32 decisions past the full buffer, 4.0e6 samples, 621).  Every
+// thread of the block calls it, after a barrier.
+template <int MODE, int REC, int MAP, int REF, class Entry>
+__device__ __forceinline__ void take_bits(const EdgeArgs& a, const TileDev& td, int words, double lam, float lamf,
+                                          const Entry& entry) {
+  const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  unsigned* bits = a.left_bits + (size_t)blockIdx.x * a.max_pairs * words;
+  for (int k = threadIdx.x >> 5; k < (td.q1 - td.q0) * words; k += nwarp) {
+    const unsigned m = bits[k];
+    if (!m) continue;
+    __syncwarp();  // every lane has read the word
+    if (lane == 0) bits[k] = 0u;
+    const int q = td.q0 + k / words, p = a.pp[q].p;
+    float x[kAcc + 2] = {};
+    if (m >> lane & 1u) {
+      const int li = k % words * 32 + lane;
+      exact_eval<MODE, REC, MAP, REF>(a, entry(q, p, li), td.begin + li, lam, lamf, [&](int slot, float v) { x[slot] = v; });
+    }
+    // reduce-scatter: lane L ends with the sum of slot L >> 2
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+    double k4[4], k2[2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      k4[i] = (double)(b4 ? x[4 + i] : x[i]) + (double)__shfl_xor_sync(0xffffffffu, b4 ? x[i] : x[4 + i], 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) k2[i] = (b3 ? k4[2 + i] : k4[i]) + __shfl_xor_sync(0xffffffffu, b3 ? k4[i] : k4[2 + i], 8);
+    double sum = (b2 ? k2[1] : k2[0]) + __shfl_xor_sync(0xffffffffu, b2 ? k2[0] : k2[1], 4);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    if ((lane & 3) == 0 && sum != 0.0) atomicAdd(a.pair_acc + (size_t)kAcc * p + (lane >> 2), sum);
+    if constexpr (REF && MODE != MODE_FWD) {
+      double f = (double)(b4 ? x[9] : x[8]) + (double)__shfl_xor_sync(0xffffffffu, b4 ? x[8] : x[9], 16);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+      if ((lane & 15) == 0 && f != 0.0) atomicAdd(a.pair_facc + 2 * (size_t)p + (lane >> 4), f);
     }
   }
 }
@@ -229,6 +295,15 @@ __device__ void exact_eval(const EdgeArgs& a, const AmbEntry& en, int64_t rec, d
 // refine scene.
 template <int REF>
 __host__ __device__ constexpr int edge_slots() { return REF ? kAcc + 2 : kAcc; }
+
+// k_edge's samples left in the block's bits; X, UV: the staged records of work item t.
+template <int MODE, int REC, int MAP, int REF>
+__device__ __noinline__ void exact_eval_left(const EdgeArgs& a, int t, int words, const float4* X, const float2* UV,
+                                             double lam, float lamf) {
+  const TileDev td = a.tiles[t];
+  take_bits<MODE, REC, MAP, REF>(a, td, words, lam, lamf,
+                                 [&](int q, int p, int li) { return AmbEntry{UV[li].x, UV[li].y, X[li].z, p, q}; });
+}
 
 template <int MODE, int REC, int MAP, int GATHER, int RPT, int REF>
 __global__ void __launch_bounds__(512) k_edge(EdgeArgs a) {
@@ -316,7 +391,6 @@ __global__ void __launch_bounds__(512) k_edge(EdgeArgs a) {
       if (!pact.y) continue;  // uniform over the block
       const int p = pact.x;
       const PairParam P = a.pp[q];
-      const float Wm1 = (float)(P.W - 1), Hm1 = (float)(P.H - 1);
       float acc[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) acc[k] = 0.f;
@@ -413,23 +487,10 @@ __global__ void __launch_bounds__(512) k_edge(EdgeArgs a) {
                 const float2 uv = s_UV[li];  // refine scenes: reloaded from the record
                 s_amb[pos] = AmbEntry{uv.x, uv.y, s_X[li].z, p, q};
                 if constexpr (REF) s_amb_rec[pos] = td.begin + li;
-              } else {
-                // buffer full: evaluate this sample with FP32 decisions instead
-                atomicAdd(a.q_overflow, 1u);
-                ok[r] = (Y2[r] > eps_z) && (up[r] >= 0.f) && (up[r] <= Wm1) && (vp[r] >= 0.f) && (vp[r] <= Hm1);
-                if (ok[r]) {
-                  const int fx0 = min(max(x0[r], 0), P.W - 2), fy0 = min(max(y0[r], 0), P.H - 2);
-                  const float fa = up[r] - (float)fx0, fb = vp[r] - (float)fy0;
-                  float n00, n01, n10, n11;
-                  taps<MAP, GATHER>(a.map, P.map_off, P.pitch, P.tex, fx0, fy0, n00, n01, n10, n11);
-                  const float t2 = fmaf(fa, n01 - n00, n00);
-                  const float b2 = fmaf(fa, n11 - n10, n10);
-                  d = fmaf(fb, b2 - t2, t2);
-                  ddu = fmaf(fb, (n11 - n10) - (n01 - n00), n01 - n00);
-                  ddv = b2 - t2;
-                }
               }
             }
+            if (base + __popc(bal) > kAmbCap)  // uniform over the warp
+              leave_bits(a, RPT * nwarp, q - pb, (g + r) * nwarp + warp, bal, kAmbCap - base, lane);
           }
           float dzs = 0.f;  // refine, fused pass: the sample's d(rho)/dz (0 unless valid)
           if (ok[r]) {
@@ -500,7 +561,7 @@ __global__ void __launch_bounds__(512) k_edge(EdgeArgs a) {
     __syncthreads();  // every warp has stored its partial sums for this tile
     // the exact-path count is read between the two barriers: every append of this tile is done,
     // and no warp appends for the next tile before the second one
-    const int n_amb = min(s_amb_n, kAmbCap);
+    const int n_all = s_amb_n, n_amb = min(n_all, kAmbCap);
     // flush: warps summed in a fixed order, one FP64 atomic per used pair slot
     constexpr int S0 = MODE == MODE_BWD ? 2 : 0;
     constexpr int NS = MODE == MODE_FWD ? 2 : NSLOT - S0;
@@ -522,9 +583,10 @@ __global__ void __launch_bounds__(512) k_edge(EdgeArgs a) {
     // exact path: when the buffer holds more than kAmbRun entries, and once more before exiting
     if (n_amb > (s_tile < a.n_tiles ? kAmbRun : 0)) {
       for (int k = threadIdx.x; k < n_amb; k += blockDim.x) exact_eval<MODE, REC, MAP, REF>(a, s_amb[k], REF ? s_amb_rec[k] : (int64_t)0, lam64, lam);
+      if (n_all > kAmbCap) exact_eval_left<MODE, REC, MAP, REF>(a, t, RPT * nwarp, s_X, s_UV, lam64, lam);
       __syncthreads();
       if (threadIdx.x == 0) {
-        atomicAdd(a.q_count, (unsigned)n_amb);
+        atomicAdd(a.q_count, (unsigned)n_all);
         s_amb_n = 0;
       }
       __syncthreads();
@@ -579,15 +641,6 @@ __global__ void __launch_bounds__(512) k_edge(EdgeArgs a) {
 #else
 #define EPO_POSE_BOUNDS __maxnreg__(56)
 #endif
-// The exact path for one buffered sample of a pose-only scene, reloading its record (a call,
-// not inlined, so that its FP64 registers do not count against the kernel's).
-template <int MODE, int REC, int MAP>
-__device__ __noinline__ void exact_eval_rec(const EdgeArgs& a, int64_t rec, int p, int q, double lam, float lamf) {
-  float u, v, z;
-  load_record<REC>(a.rec, rec, u, v, z);
-  exact_eval<MODE, REC, MAP, 0>(a, AmbEntry{u, v, z, p, q}, (int64_t)0, lam, lamf);
-}
-
 // An ambiguous sample of the pose kernel: its record and PairParam; the exact path reloads the
 // record (rare), so that the kernel keeps no copy of the raw pixels in shared memory.
 struct AmbRef {
@@ -602,6 +655,24 @@ struct AmbRef {
 #endif
 constexpr int kAmbCapPose = EPO_POSE_AMBCAP;
 constexpr int kAmbRunPose = kAmbCapPose * 3 / 8;
+
+// The exact path of a block: its n buffered samples, then those of work item t left in its bits.
+template <int MODE, int REC, int MAP>
+__device__ __noinline__ void exact_pass(const EdgeArgs& a, const AmbRef* amb, int n, int t, int words, double lam, float lamf) {
+  for (int k = threadIdx.x; k < min(n, kAmbCapPose); k += blockDim.x) {
+    const AmbRef ar = amb[k];
+    float u, v, z;
+    load_record<REC>(a.rec, ar.rec, u, v, z);
+    exact_eval<MODE, REC, MAP, 0>(a, AmbEntry{u, v, z, a.pp[ar.q].p, ar.q}, (int64_t)0, lam, lamf);
+  }
+  if (n <= kAmbCapPose) return;
+  const TileDev td = a.tiles[t];
+  take_bits<MODE, REC, MAP, 0>(a, td, words, lam, lamf, [&](int q, int p, int li) {
+    float u, v, z;
+    load_record<REC>(a.rec, td.begin + li, u, v, z);
+    return AmbEntry{u, v, z, p, q};
+  });
+}
 
 // HALVES = 2 (four records per thread): the block does the work item of one twice as wide with two
 // records per thread, in the same order.  Thread t is its threads t and t + blockDim in turn: the
@@ -702,8 +773,7 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
           // beyond t = 1/4 (or NaN) the bound is not relied on: the exact path decides
           const bool guard = !(tb[r] <= 0.25f);
           // the footprint is fetched wherever FP32 says the sample is valid; it is accumulated
-          // where no decision is in doubt (and, should the exact path's buffer be full, where
-          // FP32 says valid)
+          // where no decision is in doubt
           fetch[r] = dz > 0.f && in_cell;
           ok[r] = fetch[r] && dz > E && !near && !guard;
           // candidates for the exact path; whether they are near the image is checked on the
@@ -777,15 +847,10 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
             if (qa[r]) {
               const int pos = base + __popc(bal & lanemask_lt);
               const int li = threadIdx.x + at(g, r) * blockDim.x;
-              if (pos < kAmbCapPose) {
-                s_amb[pos] = AmbRef{td.begin + li, q, 0};
-              } else {
-                // buffer full (a tile with hundreds of samples on cell lines): the sample keeps
-                // its FP32 decisions, counted in q_overflow
-                atomicAdd(a.q_overflow, 1u);
-                use[r] = fetch[r];
-              }
+              if (pos < kAmbCapPose) s_amb[pos] = AmbRef{td.begin + li, q, 0};
             }
+            if (base + __popc(bal) > kAmbCapPose)  // uniform over the warp
+              leave_bits(a, RPT * nwarp, q - pb, at(g, r) * nwarp + warp, bal, kAmbCapPose - base, lane);
           }
         }
 #pragma unroll
@@ -833,7 +898,7 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
     __syncthreads();  // every warp has stored its partial sums and appended its exact-path samples
     // the exact-path counts are read between the two barriers: every append of this tile is
     // done, and no warp appends for the next tile before the second one
-    const int n_amb = min(s_amb_n, kAmbCapPose);
+    const int n_all = s_amb_n, n_amb = min(n_all, kAmbCapPose);
     constexpr int S0 = MODE == MODE_BWD ? 2 : 0;
     constexpr int NS = MODE == MODE_FWD ? 2 : kAcc - S0;
     const int nq = (pe - pb) * NS;
@@ -848,13 +913,10 @@ __global__ void EPO_POSE_BOUNDS k_edge_pose(EdgeArgs a) {
     if (threadIdx.x == 0) s_tile = s_next;
     __syncthreads();
     if (n_amb > (s_tile < a.n_tiles ? kAmbRunPose : 0)) {
-      for (int k = threadIdx.x; k < n_amb; k += blockDim.x) {
-        const AmbRef ar = s_amb[k];
-        exact_eval_rec<MODE, REC, MAP>(a, ar.rec, a.pp[ar.q].p, ar.q, lam64, lam);
-      }
+      exact_pass<MODE, REC, MAP>(a, s_amb, n_all, t, RPT * nwarp, lam64, lam);
       __syncthreads();
       if (threadIdx.x == 0) {
-        atomicAdd(a.q_count, (unsigned)n_amb);
+        atomicAdd(a.q_count, (unsigned)n_all);
         s_amb_n = 0;
       }
       __syncthreads();

@@ -159,9 +159,10 @@ struct EdgeArgs {
   double* pair_acc;              // n_pairs x kAcc
   const double* lambda;          // device scalar
   unsigned int* q_count;         // samples re-evaluated on the exact path this evaluation
-  unsigned int* q_overflow;      // samples that found the block buffer full (FP32 decisions)
+  unsigned int* left_bits;       // per block, pair of its item and 32 records: the samples that found
+                                 // the block's buffer full (all zero between launches)
   int* tile_counter;             // dynamic work distribution, reset by the pair setup
-  int32_t max_pairs;             // most outgoing pairs of any view (shared accumulators)
+  int32_t max_pairs;             // most pairs of one work item (shared accumulators, left_bits)
   float delta;
   float eps_z;
   // focal and depth refinement (scenes created with refine = 1; Eqs. 4-5)
