@@ -1942,8 +1942,10 @@ epo_status epo_set_pair_subset(epo_scene_t S, int32_t n, const int32_t* ids) {
 // thermal drift during tuning affects all of them alike, and each candidate is judged by
 // the median of its launches. A first pass over all candidates (3 timed launches each)
 // keeps the 4 best; with tail_pairs = -1 each of those is also tried with its last wave
-// split into items of 2 pairs and of 1 pair, and 12 further passes decide.  (Every item split
-// by pairs, tail_pairs <= -2, was never faster on the benchmark workloads: not a candidate.)
+// split into items of 2 pairs and of 1 pair, and 12 further passes decide.  The schedule the
+// scene has (default_schedule's, with its split of every item and its two-halves form) is a
+// candidate of both rounds, so that tuning does not end with a slower one: without it, views of
+// 200x150 with all pairs ended 17 % (10 views), 13 % (16) and 10 % (20) above the default.
 epo_status epo_autotune(epo_scene_t S) {
   EPO_RANGE("epo_autotune");
   if (!S) return fail(S, EPO_ERR_INVALID_ARG, "null scene");
@@ -1966,6 +1968,9 @@ epo_status epo_autotune(epo_scene_t S) {
         if (!schedule_fits(S, sc)) continue;
         cands.push_back({sc, {}, 0.f});
       }
+  const Sched own = S->sch;
+  const auto is_own = [&](const Cand& c) { return c.sc == own; };
+  if (schedule_fits(S, own) && std::none_of(cands.begin(), cands.end(), is_own)) cands.push_back({own, {}, 0.f});
   if (cands.empty()) return fail(S, EPO_ERR_INVALID_ARG, "no edge-kernel schedule fits this scene");
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
@@ -2019,7 +2024,12 @@ epo_status epo_autotune(epo_scene_t S) {
   if (st == EPO_OK) {
     for (auto& c : cands) c.med = median(c.ms);
     std::stable_sort(cands.begin(), cands.end(), [](const Cand& x, const Cand& y) { return x.med < y.med; });
-    if (cands.size() > 4) cands.resize(4);
+    if (cands.size() > 4) {
+      const auto o = std::find_if(cands.begin() + 4, cands.end(), is_own);  // stays whatever its place
+      const bool fifth = o != cands.end();
+      if (fifth) cands[4] = *o;
+      cands.resize(fifth ? 5 : 4);
+    }
     if (S->opt.tail_pairs == -1) {
       const size_t n4 = cands.size();
       for (size_t k = 0; k < n4; ++k)
@@ -2027,7 +2037,7 @@ epo_status epo_autotune(epo_scene_t S) {
           Cand c = cands[k];
           c.sc.tail = t;
           c.ms.clear();
-          cands.push_back(c);
+          if (schedule_fits(S, c.sc)) cands.push_back(c);
         }
       for (size_t k = n4; k < cands.size() && st == EPO_OK; ++k) st = launch(cands[k], false);  // warm-up
     }
