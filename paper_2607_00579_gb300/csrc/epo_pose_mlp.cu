@@ -70,23 +70,12 @@ __device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_g
 template <int N>  // until at most the N youngest groups are in flight
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// 1 / x and 1 / sqrt(x) for x > 0: the FP32 approximation refined by two FP64 Newton steps (relative
-// error below 2^-50); outside FP32's range the operations themselves.
-__device__ __forceinline__ double rcp64(double x) {
-  if (!(x > 1e-30 && x < 1e30)) return 1.0 / x;
-  float rf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"((float)x));
-  double r = (double)rf;
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
-__device__ __forceinline__ double rsqrt64(double x) {
-  if (!(x > 1e-30 && x < 1e30)) return 1.0 / sqrt(x);
-  float rf;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"((float)x));
-  double r = (double)rf;
-  r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
-  return fma(0.5 * r, fma(-x * r, r, 1.0), r);
+// x / d of a warp-uniform vector x: one division for the three (an FP64 instruction costs a warp the
+// same for one lane as for 32).  Every lane calls it.
+__device__ __forceinline__ void div3(const double* x, double d, double* q, int lane) {
+  const double y = (lane == 0 ? x[0] : (lane == 1 ? x[1] : x[2])) / d;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) q[r] = __shfl_sync(0xffffffffu, y, r);
 }
 
 // Sums of 8 values over a warp, the butterfly over lane distances 16, 8, 4, 2, 1 as a reduce-scatter:
@@ -108,6 +97,25 @@ __device__ __forceinline__ void cross3(const double* a, const double* b, double*
   c[0] = a[1] * b[2] - a[2] * b[1];
   c[1] = a[2] * b[0] - a[0] * b[2];
   c[2] = a[0] * b[1] - a[1] * b[0];
+}
+
+// phi: Gram-Schmidt on the first two columns a1, a2 of a 3x4 matrix P, b1 = a1 / n1, b2 = u2 / n2 with
+// u2 = a2 - c b1, c = b1 . a2.  Warp-uniform; every lane calls it.
+struct Phi {
+  double a2[3], b1[3], b2[3], n1, n2, c;
+};
+__device__ __forceinline__ void gram_schmidt(const double* P, Phi& f, int lane) {
+  const double a1[3] = {P[0], P[4], P[8]};
+  f.n1 = sqrt(dot3(a1, a1));
+  div3(a1, f.n1, f.b1, lane);
+  double u2[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) f.a2[r] = P[4 * r + 1];
+  f.c = dot3(f.b1, f.a2);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) u2[r] = f.a2[r] - f.c * f.b1[r];
+  f.n2 = sqrt(dot3(u2, u2));
+  div3(u2, f.n2, f.b2, lane);
 }
 
 }  // namespace
@@ -200,22 +208,17 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_forward(StepArgs a, int cha
   }
   __syncwarp();
   double* Ts = a.T_store + 12 * (size_t)v;
+  Phi f;
+  gram_schmidt(s_Pp, f, lane);
   if (lane == 0) {
-    // phi: Gram-Schmidt on the first two columns; the offset delta (FP64)
+    // the pose: phi's columns and the offset delta (FP64)
     const double* Pp = s_Pp;
-    const double a1[3] = {Pp[0], Pp[4], Pp[8]}, a2[3] = {Pp[1], Pp[5], Pp[9]};
-    const double r1 = rsqrt64(dot3(a1, a1));
-    const double b1[3] = {a1[0] * r1, a1[1] * r1, a1[2] * r1};
-    const double c = dot3(b1, a2);
-    const double u2[3] = {a2[0] - c * b1[0], a2[1] - c * b1[1], a2[2] - c * b1[2]};
-    const double r2 = rsqrt64(dot3(u2, u2));
-    const double b2[3] = {u2[0] * r2, u2[1] * r2, u2[2] * r2};
     double b3[3];
-    cross3(b1, b2, b3);
+    cross3(f.b1, f.b2, b3);
     bool finite = true;
     for (int r = 0; r < 3; ++r) {
-      s_T[4 * r] = b1[r];
-      s_T[4 * r + 1] = b2[r];
+      s_T[4 * r] = f.b1[r];
+      s_T[4 * r + 1] = f.b2[r];
       s_T[4 * r + 2] = b3[r];
       s_T[4 * r + 3] = Pp[4 * r + 3] + sc_s * (double)a.mlp_delta[3 * (size_t)v + r];
     }
@@ -269,49 +272,49 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_backward(StepArgs a) {
 #pragma unroll
     for (int l = 0; l < 5; ++l) z[l] = zs[l * H + j];
   }
+  Phi f;
+  if (j < 32) gram_schmidt(a.mlp_Pp + 12 * (size_t)v, f, j);
   griddep_wait();  // the poses' gradient
-  if (j == 0) {
+  if (j < 32) {
     // G = (g_v, g_w) at T = P^s: dL/dt = g_v, and (for the tangent dR = [w]x R that phi
-    // produces) dL/dR = 1/2 [g_w + g_v x t]x R; then back through Gram-Schmidt (FP64), whose
-    // orthonormal columns are those of T
+    // produces) dL/dR = 1/2 [g_w + g_v x t]x R; then back through Gram-Schmidt (FP64)
     const double* G = a.grad + 6 * (size_t)v;
     const double* T = a.T_store + 12 * (size_t)v;
-    const double* Pp = a.mlp_Pp + 12 * (size_t)v;
     const double gv[3] = {G[0], G[1], G[2]}, t[3] = {T[3], T[7], T[11]};
     double w[3];
     cross3(gv, t, w);
     for (int r = 0; r < 3; ++r) w[r] = 0.5 * (w[r] + G[3 + r]);
-    const double b1[3] = {T[0], T[4], T[8]}, b2[3] = {T[1], T[5], T[9]}, b3[3] = {T[2], T[6], T[10]};
-    const double a1[3] = {Pp[0], Pp[4], Pp[8]}, a2[3] = {Pp[1], Pp[5], Pp[9]};
-    const double r1 = rcp64(dot3(a1, b1));  // 1 / |a1|
-    const double c = dot3(b1, a2);
-    const double r2 = rcp64(dot3(a2, b2));  // 1 / |a2 - c b1|
+    const double r1[3] = {T[0], T[4], T[8]}, r2[3] = {T[1], T[5], T[9]}, r3[3] = {T[2], T[6], T[10]};
     // columns of dL/dR = [w]x R
     double g1[3], g2[3], g3[3];
-    cross3(w, b1, g1);
-    cross3(w, b2, g2);
-    cross3(w, b3, g3);
+    cross3(w, r1, g1);
+    cross3(w, r2, g2);
+    cross3(w, r3, g3);
     double x[3];
-    cross3(b2, g3, x);  // b3 = b1 x b2
+    cross3(f.b2, g3, x);  // b3 = b1 x b2
     for (int r = 0; r < 3; ++r) g1[r] += x[r];
-    cross3(g3, b1, x);
+    cross3(g3, f.b1, x);
     for (int r = 0; r < 3; ++r) g2[r] += x[r];
-    const double p2 = dot3(g2, b2);  // b2 = u2 / n2
-    double gu2[3];
-    for (int r = 0; r < 3; ++r) gu2[r] = (g2[r] - p2 * b2[r]) * r2;
-    const double q = dot3(gu2, b1);  // u2 = a2 - (b1 . a2) b1
-    double ga2[3];
+    const double p2 = dot3(g2, f.b2);  // b2 = u2 / n2
+    double gu2[3], ga1[3], ga2[3];
+    for (int r = 0; r < 3; ++r) x[r] = g2[r] - p2 * f.b2[r];
+    div3(x, f.n2, gu2, j);
+    const double q = dot3(gu2, f.b1);  // u2 = a2 - (b1 . a2) b1
     for (int r = 0; r < 3; ++r) {
-      ga2[r] = gu2[r] - q * b1[r];
-      g1[r] -= q * a2[r] + c * gu2[r];
+      ga2[r] = gu2[r] - q * f.b1[r];
+      g1[r] -= q * f.a2[r] + f.c * gu2[r];
     }
-    const double p1 = dot3(g1, b1);  // b1 = a1 / n1
-    for (int r = 0; r < 3; ++r) {
-      s_dy[4 * r] = (float)((g1[r] - p1 * b1[r]) * r1);
-      s_dy[4 * r + 1] = (float)ga2[r];
-      s_dy[4 * r + 2] = 0.f;  // the third column does not reach phi
-      s_dy[4 * r + 3] = (float)(a.mlp_scale[sc] * gv[r]);  // the translation output is scaled by s
-      a.mlp_gdelta[3 * (size_t)v + r] = s_dy[4 * r + 3];
+    const double p1 = dot3(g1, f.b1);  // b1 = a1 / n1
+    for (int r = 0; r < 3; ++r) x[r] = g1[r] - p1 * f.b1[r];
+    div3(x, f.n1, ga1, j);
+    if (j == 0) {
+      for (int r = 0; r < 3; ++r) {
+        s_dy[4 * r] = (float)ga1[r];
+        s_dy[4 * r + 1] = (float)ga2[r];
+        s_dy[4 * r + 2] = 0.f;  // the third column does not reach phi
+        s_dy[4 * r + 3] = (float)(a.mlp_scale[sc] * gv[r]);  // the translation output is scaled by s
+        a.mlp_gdelta[3 * (size_t)v + r] = s_dy[4 * r + 3];
+      }
     }
   }
   stage_wait<3>();
