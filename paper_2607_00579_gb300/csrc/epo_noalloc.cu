@@ -61,18 +61,6 @@ constexpr int kNaMaxDevices = 64;
 NaScratch* g_scratch_ptr[kNaMaxDevices] = {};
 std::mutex g_scratch_mutex;
 
-// 1 / x for a finite x > 0: the FP32 approximate reciprocal refined by two FP64 Newton steps
-// (relative error below 2^-51); a correctly rounded FP64 division costs twice the instructions.
-// Outside FP32's range the division itself.
-__device__ __forceinline__ double rcp64(double x) {
-  if (!(x > 1e-30 && x < 1e30)) return 1.0 / x;
-  float rf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"((float)x));
-  double r = (double)rf;
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
-
 // 16 lanes per pair: lanes 0..8 one entry of R_ji each, lanes 9..11 one of t_ji.
 constexpr int kNaSetupThreads = 64;
 
@@ -280,7 +268,9 @@ __global__ void __launch_bounds__(kNaThreads, 4) k_na_edge(epo_noalloc_problem p
     // lane 3r + c < 9: B[r][c] = f_r M[r][c] + c_r M[2][c], M = R K_i^-1, (f, c)_r = (fx_j, cx_j),
     // (fy_j, cy_j), (1, 0); lane 9 + r: c[r] = f_r t[r] + c_r t[2]
     const int e = min(lane, 11), r = e < 9 ? e / 3 : e - 9, c = e % 3;
-    const double rx = rcp64(s_Ki[0]), ry = rcp64(s_Ki[1]);
+    // the four reciprocals in one division: 1 / focal length of view i (lanes 0, 1) and view j (2, 3)
+    const double rf = 1.0 / (lane & 2 ? s_Kj : s_Ki)[lane & 1];
+    const double rx = __shfl_sync(0xffffffffu, rf, 0), ry = __shfl_sync(0xffffffffu, rf, 1);
     const auto entry = [&](int row) {
       if (e >= 9) return q.t[row];
       const double* R = q.R + 3 * row;
@@ -308,7 +298,7 @@ __global__ void __launch_bounds__(kNaThreads, 4) k_na_edge(epo_noalloc_problem p
     } else if (lane == 12 || lane == 13) {
       (lane == 12 ? s_f.cx : s_f.cy) = split(s_Kj[lane - 10]);
     } else if (lane == 14 || lane == 15) {
-      (lane == 14 ? s_f.rfx : s_f.rfy) = split(rcp64(s_Kj[lane - 14]));
+      (lane == 14 ? s_f.rfx : s_f.rfy) = split(rf);
     }
   }
   __syncthreads();
@@ -381,7 +371,7 @@ __global__ void __launch_bounds__(kNaFinThreads) k_na_finish(epo_noalloc_problem
     double part = 0.0;
     for (int p = threadIdx.x; p < P; p += kNaFinThreads) {
       const double denom = S->acc[p][slot];
-      if (denom > 0.0) part += S->acc[p][0] * rcp64(denom);
+      if (denom > 0.0) part += S->acc[p][0] / denom;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
@@ -422,7 +412,7 @@ __global__ void __launch_bounds__(kNaFinThreads) k_na_finish(epo_noalloc_problem
         const double* a = S->acc[q];
         const double denom = a[slot];
         if (denom > 0.0) {
-          const double c = w2 * rcp64(denom);
+          const double c = w2 / denom;
           const double ga0 = c * a[2], ga1 = c * a[3], ga2 = c * a[4], gb0 = c * a[5], gb1 = c * a[6], gb2 = c * a[7];
           if (src) {
             // source view: -Ad(T_ji)^T (ga, gb) = (-R^T ga, R^T (t x ga) - R^T gb)
