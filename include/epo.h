@@ -126,10 +126,12 @@ typedef struct {
   int32_t tail_pairs;        /* work items of the last wave (as many as the grid has blocks):
                                 0 = each covers all of its view's pairs, like the others;
                                 n > 0 = split into items of at most n pairs, so that the
-                                blocks finish together; -1 = default (autotuned when
-                                autotune is on, else chosen from the amount of work);
-                                n <= -2 = every work item, not
-                                only the last wave's, covers at most -n pairs */
+                                blocks finish together; -1 = default: autotuned when
+                                autotune is on; else chosen from the amount of work where
+                                the gather is EPO_GATHER_TEX (or AUTO), grid_blocks is 0 and
+                                the schedule is the default one or, without refinement, 128
+                                threads with four records each; else 0.  n <= -2 = every
+                                work item, not only the last wave's, covers at most -n pairs */
   int32_t refine;            /* 1: the scene also carries the focal and depth refinement of
                                 Section 3 (Eq. 4: f_i = f_i^0 (1 + gamma_i) for both focal
                                 lengths of view i; Eq. 5: every edge pixel's depth is
@@ -181,7 +183,9 @@ typedef struct {
   int32_t gather, block_threads, records_per_thread, grid_blocks; /* schedule in use */
   int32_t kernels_per_step;  /* kernel launches in one epo_step */
   int32_t tail_pairs;        /* pairs per work item of the last wave (0 = not split; a
-                                negative n: every work item covers at most -n pairs) */
+                                negative n: every work item covers at most -n pairs).  -1, one
+                                pair each, is the library's choice: given as an option it asks
+                                for the default */
 } epo_scene_info;
 
 /* Defaults: delta 1, lambda 10 -> 6 over 1000 steps, eps_z 1e-6, NORM_VALID,
@@ -453,7 +457,11 @@ epo_status epo_gather_probe(int32_t n_maps, int32_t W, int32_t H, int32_t map_dt
  *
  * It computes what epo_loss_and_grad_dev computes (Eqs. 6-8 and the
  * left-perturbation pose gradient, EPO_F32 records and FP32 maps) for one
- * scene, with every projection and branch decision taken in FP64.  The
+ * scene.  Every branch decision is the one of an FP64 evaluation, and every
+ * projected position is within 2^-29 of a pixel of it before the value and
+ * slope terms are formed in FP32 (positions are carried as pairs of floats
+ * beside a bound on their error, and in FP64 where that is wider or a
+ * decision lies within it).  The
  * intermediate per-pair sums live in one file-scope device array of the
  * library of fixed size: EPO_NOALLOC_MAX_PAIRS x 21 doubles = 688,128
  * bytes (672 KiB), which every GPU that loads the library reserves until

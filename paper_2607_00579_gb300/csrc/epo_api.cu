@@ -598,7 +598,7 @@ bool schedule_fits(epo_scene* S, const Sched& sc) {
 // What the options leave to the library of a scene's schedule (texture gather, the library's grid).  A
 // split by pairs moves whole sums to other blocks, and the two forms of the default item (512 records,
 // two per thread of 256 threads or four per thread of 128 in two halves, k_edge_pose) form the same
-// sums, so all of these give the same bits as the unsplit 256-thread form.
+// FP32 sums, so all of these differ from the unsplit 256-thread form in the order of FP64 additions only.
 //
 // With U = work items x pairs (those a step evaluates) and G = the resident 128-thread blocks:
 //  - no block size given and U < 4 G: 256 threads; one wave of items if at most 4 pairs each make one

@@ -19,7 +19,9 @@
 // FMA products) beside a bound on their error; a sample whose bound is too wide, or that has a
 // decision within it, takes the FP64 form (sample_exact).  The final gather is a warp per pose; it
 // was one block that scanned every pair for every pose.  24 views of 256x192, 192 pairs, 0.57 M
-// evaluations: 200 us for the call (edge kernel 104, gather 98) before, 26 us now.
+// evaluations: 200 us for the call (edge kernel 104, gather 98) before, 26 us now.  Over 100 drawn
+// scenes the gradient is as far from a 64-bit evaluation of everything as with FP64 positions: median 3.035e-8
+// of its norm both ways, largest 7.349e-8 (the FP32 terms and sums).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

@@ -21,7 +21,8 @@
 // shared memory with cp.async, all but one of the hidden layers at once, so that the layers wait for
 // one trip to L2 and not for one each; backward starts them while the pose kernel still runs
 // (programmatic launch) and forms the FP64 part meanwhile.  32 views, one scene, warm caches:
-// forward 29-32 -> 12 us, backward 19.6 -> 13, update 17 -> 8; a step with its read-backs 172 -> 131.
+// forward 29-32 -> 12.6 us, backward 19.6 -> 14.6 (its roots run before the wait, beside the pose kernel),
+// update 17 -> 8; a step with its read-backs 172 -> 131.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
