@@ -73,3 +73,30 @@ def test_records_beyond_the_stated_maximum_are_left_out():
     o = oracle.OracleScene(sc.W, sc.H, sc.K, np.arange(4, dtype=np.int64) * 256, sc.rec[keep],
                            [m.astype(np.float64) for m in maps], sc.pairs).loss_grad(sc.T_init, lam=10.0)
     check_against_oracle(got_loss, got_grad, o, sc.pairs, sc.T_init)
+
+
+def test_views_of_different_sizes():
+    """Each target's own width, height, intrinsics and map offset."""
+    r = np.random.default_rng(8)
+    W, H = np.array([70, 33, 128, 9, 61], np.int32), np.array([50, 90, 17, 12, 47], np.int32)
+    n = len(W)
+    off = np.concatenate([[0], np.cumsum([300, 513, 40, 256, 700])]).astype(np.int64)
+    rec = np.zeros((off[-1], 4), np.float32)
+    for v in range(n):
+        part = rec[off[v]:off[v + 1]]
+        part[:, 0], part[:, 1] = r.integers(0, W[v], len(part)), r.integers(0, H[v], len(part))
+    rec[:, 2] = r.uniform(2, 5, len(rec))
+    T = np.zeros((n, 3, 4))
+    for v in range(n):
+        T[v, :, :3] = synth._rotvec_to_matrix(r.normal(0, 0.03, 3))
+        T[v, :, 3] = r.normal(0, 0.1, 3)
+    K = np.stack([1.1 * W, 1.05 * H, W / 2 + 0.3, H / 2 - 0.7], axis=1)
+    maps = [(2.5 + 2 * np.sin(np.arange(w) / 6 + v)[None, :] + 2 * np.cos(np.arange(h) / 5)[:, None]).clip(0).astype(np.float32)
+            for v, (w, h) in enumerate(zip(W, H))]
+    pairs = np.array([(a, b) for a in range(n) for b in range(n) if a != b], np.int32)
+    sc = synth.Scene(W=W, H=H, K=K, T_gt=T.reshape(n, 12), T_init=T.reshape(n, 12), rec_off=off, rec=rec, edges=[],
+                     pairs=pairs, fixed=np.zeros(n, np.uint8), scale=1.0, depth_gt_at_rec=np.zeros(len(rec)))
+    got_loss, got_grad = Problem(sc, maps)(sc.T_init, B.EPO_NORM_VALID)
+    o = oracle.scene_from_synth(sc, [m.astype(np.float64) for m in maps]).loss_grad(sc.T_init, lam=10.0)
+    assert o["pair_stats"][:, 1].min() > 0
+    check_against_oracle(got_loss, got_grad, o, sc.pairs, sc.T_init)
